@@ -101,37 +101,6 @@ template <int BYTES> __device__ __forceinline__ void cp_async_zfill(void *smem, 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Programmatic dependent launch (sm_90 and later).  The passes of an apply are
-// launched with programmatic stream serialization: each pass kernel triggers its
-// dependents as its blocks start, so once the last wave of a pass is resident
-// the next pass's blocks may be scheduled into the slots that free up; they wait
-// (griddepcontrol.wait) for the previous grid to complete and its memory to be
-// visible before their first global access.  Launched without the attribute,
-// both instructions are no-ops.
-__device__ __forceinline__ void pdl_wait_and_trigger()
-{
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
-
-// A failed launch sets the runtime's last error, which every apply checks after
-// its launches (cudaGetLastError), as for <<<>>> launches.
-template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
-{
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // xfwd: w_f of one grid row per line, FFT along x (pruned), 4 fields in turn.
 template <typename R, int L>
 __global__ void __launch_bounds__(256) k2_xfwd(const typename cplx_of<R>::type *__restrict__ x,

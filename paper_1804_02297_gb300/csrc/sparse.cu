@@ -17,15 +17,11 @@
 // Each node keeps G = [F11^{-1}; F21 F11^{-1}] (front x own) and X = F11^{-1} F12,
 // in the factor's precision or (SPM_C64H) as binary16 pairs scaled per column by
 // the column's largest component, which halves the bytes every solve reads.
-// Solve, one batched pass per tree level:
-//   forward (deepest level first): [y; t] = G w_own, w_own = y, w_bnd -= t
-//   backward (root first):         w_own -= X w_bnd.
-// Nodes of one level have disjoint own unknowns; their boundaries lie on
-// shallower separators, so one launch handles a whole level.  Dense front
+// Solve, one launch per tree level and direction (k_nd_level): nodes of one level
+// have disjoint own unknowns, and their boundaries lie on shallower separators.  Dense front
 // work (dense.cu): F11^{-1} by Gauss-Jordan with partial pivoting, then
 // X = F11^{-1} F12, F21 F11^{-1} and the update F22 - F21 X as complex GEMMs;
-// assembly, extend-add, the batched level GEMVs, gathers and scatters are
-// kernels here.
+// assembly, extend-add and the solve's levels are kernels here.
 #include <cuda_fp16.h>
 
 #include <algorithm>
@@ -297,98 +293,184 @@ template <typename C> __global__ void k_zero(C *a, long cnt)
 
 inline unsigned blocks(long cnt, int t = 256) { return (unsigned)((cnt + t - 1) / t); }
 
-// n x n identity in a column-major block with leading dimension ld
-template <typename C> __global__ void k_identity(C *a, int n, int ld)
+// ---------------------------------------------------------------- solve kernels
+// Vectors of a solve live in elimination order, [unknown u][rhs], u = D x (rank of
+// the point among all nodes' own points, in postorder) + component: a node's own
+// unknowns are contiguous and its boundary is a list of u, so a level needs no
+// packing pass.  W holds the right-hand side as it is updated, Y the solution.
+//   forward, deepest level first:  [y; t] = G w_own,  Y_own = y,  W_bnd -= t
+//   backward, root first:          Y_own -= X Y_bnd
+// One launch per level and direction.  Every node's matrix (column-major, ld rows)
+// is cut into tiles of at most ST_ROWS x ST_COLS entries; a block of 256 threads
+// owns one tile: thread t takes row t % nrow and the columns t / nrow + groups k,
+// groups = 256 / nrow, so that a tile of 49 rows keeps 245 threads busy.
+// Bound: complex64 by reading the factor; complex128 by the FP64 pipe (4 FMAs per
+// 16 bytes at 1.25 TFLOP/s: 2.5 TB/s); small grids by the 2 x levels dependent
+// launches.  Against the packing, GEMV and scatter launches this replaced (four per
+// level and direction), S^-1 Q took: 2-D n = 239 complex128 528 us (2017 before),
+// 3-D n = 32 complex64 385 us (1075 before), 16 right-hand sides 1244 us (2932).
+struct SolveTile {
+    long mat, scale;  // first entry of the tile; scale of its first column (half storage)
+    int ld, nrow, ncol;
+    int in;           // forward: unknown of the first column; backward: its place in the boundary list
+    int out, nown;    // unknown of the first row; rows that are own unknowns
+    int bout;         // place of row nown in the boundary list
+    int full;         // the tile spans every column: no other block adds to its own rows
+};
+constexpr int ST_THREADS = 256, ST_COLS = 256, ST_GROUPS = 16;
+template <typename C> constexpr int st_rows() { return 1024 / (int)sizeof(C); } // 1 KB of each column
+
+__device__ __forceinline__ float2 load_as(const float2 *p) { return __ldcs(p); }
+__device__ __forceinline__ double2 load_as(const double2 *p) { return __ldcs(p); }
+__device__ __forceinline__ float2 load_as(const __half2 *p) { return __half22float2(__ldcs(p)); }
+
+__device__ __forceinline__ void add_to(float2 *p, float2 v) { atomicAdd(p, v); }
+__device__ __forceinline__ void add_to(double2 *p, double2 v)
 {
-    long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (long)n * n) return;
-    int r = (int)(gid % n), c = (int)(gid / n);
-    a[(long)c * ld + r].x = r == c ? 1 : 0;
-    a[(long)c * ld + r].y = 0;
+    atomicAdd(&p->x, v.x);
+    atomicAdd(&p->y, v.y);
 }
 
-// Level tables.  Per node of a level: its matrix (rows x cols, column-major,
-// ld = rows) at mat_off; packed input block (cols x nrhs) at in_unit * nrhs and
-// output block (rows x nrhs) at out_unit * nrhs, in_unit / out_unit being prefix
-// sums of cols / rows over the level.
-struct LevelNode {
-    long mat_off, in_unit, out_unit, scale_off;
-    int rows, cols;
-    int own_pts, bnd_pts; // offsets into the point list
-    int nown, nbnd;
+// acc of g x over a tile's columns, NB right-hand sides.  complex64 keeps the sums
+// of g.x x and g.y x apart (two packed FP32x2 FMAs each) and joins them at the end.
+template <typename C, int NB> struct TileAcc {
+    C s[NB];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) s[b] = czero<C>();
+    }
+    __device__ __forceinline__ void mac(C g, const C *x)
+    {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) s[b] = cfma(g, x[b], s[b]);
+    }
+    __device__ __forceinline__ C get(int b) const { return s[b]; }
 };
-struct Tile {
-    int node, row0, col0;
+template <int NB> struct TileAcc<float2, NB> {
+    float2 p[NB], q[NB];
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) p[b] = q[b] = make_float2(0.f, 0.f);
+    }
+    __device__ __forceinline__ void mac(float2 g, const float2 *x)
+    {
+        const float2 gx = make_float2(g.x, g.x), gy = make_float2(g.y, g.y);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            p[b] = __ffma2_rn(gx, x[b], p[b]);
+            q[b] = __ffma2_rn(gy, x[b], q[b]);
+        }
+    }
+    __device__ __forceinline__ float2 get(int b) const { return make_float2(p[b].x - q[b].y, p[b].y + q[b].x); }
 };
-constexpr int GT_ROWS = 256, GT_COLS = 256;
 
-// out[node] += M[node][row0:+256, col0:+256] * in[node][col0:+256, :]; GT_NB
-// right-hand sides per pass over the tile (1 for a single RHS; 4, 8 or 16 for
-// blocks, by block size and precision).
-// S = C: stored as is; S = __half2: binary16 pairs, column c scaled by scale[c].
-__device__ __forceinline__ float2 load_as(const float2 *p) { return *p; }
-__device__ __forceinline__ double2 load_as(const double2 *p) { return *p; }
-__device__ __forceinline__ float2 load_as(const __half2 *p) { return __half22float2(*p); }
-
-template <typename C, int GT_NB, typename S>
-__global__ void __launch_bounds__(GT_ROWS) k_level_gemv(const S *__restrict__ M, const float *__restrict__ scales,
-                                                        const LevelNode *__restrict__ nodes,
-                                                        const Tile *__restrict__ tiles, const C *__restrict__ in,
-                                                        C *out, int nrhs)
+template <typename C, typename S, int NB, bool FWD>
+__global__ void __launch_bounds__(ST_THREADS) k_nd_level(const S *__restrict__ M, const float *__restrict__ scales,
+                                                         const SolveTile *__restrict__ tiles,
+                                                         const int *__restrict__ bnd, C *W, C *Y, int nrhs)
 {
-    using R = decltype(C{}.x);
-    __shared__ C xs[GT_COLS * GT_NB];
-    const Tile tl = tiles[blockIdx.x];
-    const LevelNode nd = nodes[tl.node];
-    const int r = tl.row0 + threadIdx.x;
-    const int ncol = min(GT_COLS, nd.cols - tl.col0);
-    const C *inb = in + nd.in_unit * nrhs;
-    C *outb = out + nd.out_unit * nrhs;
     constexpr bool SCALED = !std::is_same<S, C>::value;
-    for (int b0 = 0; b0 < nrhs; b0 += GT_NB) {
-        const int nb = min(GT_NB, nrhs - b0);
-        __syncthreads();
-        for (int i = threadIdx.x; i < GT_COLS * GT_NB; i += blockDim.x) {
-            int c = i % GT_COLS, b = i / GT_COLS;
-            C v;
-            v.x = 0;
-            v.y = 0;
-            if (c < ncol && b < nb) {
-                v = inb[(long)(b0 + b) * nd.cols + tl.col0 + c];
-                if constexpr (SCALED) {
-                    const R sc = (R)scales[nd.scale_off + tl.col0 + c];
-                    v.x *= sc;
-                    v.y *= sc;
-                }
+    constexpr int UNR = NB >= 16 ? 4 : 8; // matrix entries a thread has in flight
+    __shared__ __align__(16) C xs[(ST_COLS > ST_THREADS ? ST_COLS : ST_THREADS) * NB];
+    const SolveTile tl = tiles[blockIdx.x];
+    const int groups = min(ST_THREADS / tl.nrow, ST_GROUPS);
+    const int row = threadIdx.x % tl.nrow, g = threadIdx.x / tl.nrow;
+    const bool act = g < groups;
+    const S *mrow = M + tl.mat + row;
+    const int steps = (tl.ncol + groups - 1) / groups; // columns per thread
+    C cur[UNR];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int k = 0; k < UNR; ++k) {
+            const int c = g + (k0 + k) * groups;
+            cur[k] = act && c < tl.ncol ? load_as(mrow + (long)c * tl.ld) : czero<C>();
+        }
+    };
+    // the factor does not change: the first entries are fetched before the previous
+    // level's results are waited for
+    fetch(0);
+    pdl_wait_and_trigger();
+    for (int b0 = 0; b0 < nrhs; b0 += NB) {
+        const int nb = min(NB, nrhs - b0);
+        if (b0 > 0) {
+            __syncthreads(); // the sums of the previous group have been read
+            fetch(0);
+        }
+        for (int i = threadIdx.x; i < tl.ncol * NB; i += ST_THREADS) {
+            const int c = i / NB, b = i % NB;
+            C v = czero<C>();
+            if (b < nb) {
+                v = FWD ? __ldcg(W + (long)(tl.in + c) * nrhs + b0 + b) : __ldcg(Y + (long)bnd[tl.in + c] * nrhs + b0 + b);
+                if constexpr (SCALED) v = cscale(v, scales[tl.scale + c]);
             }
             xs[i] = v;
         }
         __syncthreads();
-        if (r < nd.rows) {
-            R ax[GT_NB], ay[GT_NB];
+        TileAcc<C, NB> acc;
+        acc.clear();
+        for (int k0 = 0; k0 < steps; k0 += UNR) {
+            C now[UNR];
 #pragma unroll
-            for (int b = 0; b < GT_NB; ++b) { ax[b] = 0; ay[b] = 0; }
-            const S *col = M + nd.mat_off + (long)tl.col0 * nd.rows + r;
-            constexpr int UNR = SCALED ? 16 : 4; // 4-byte elements: more loads in flight
-#pragma unroll UNR
-            for (int c = 0; c < ncol; ++c) {
-                const C g = load_as(col + (long)c * nd.rows);
+            for (int k = 0; k < UNR; ++k) now[k] = cur[k];
+            if (k0 + UNR < steps) fetch(k0 + UNR);
 #pragma unroll
-                for (int b = 0; b < GT_NB; ++b) {
-                    C xv = xs[b * GT_COLS + c];
-                    ax[b] += g.x * xv.x - g.y * xv.y;
-                    ay[b] += g.x * xv.y + g.y * xv.x;
-                }
+            for (int k = 0; k < UNR; ++k) {
+                const int c = g + (k0 + k) * groups;
+                if (c < tl.ncol) acc.mac(now[k], xs + c * NB);
             }
+        }
+        __syncthreads();
+        if (act) {
 #pragma unroll
-            for (int b = 0; b < GT_NB; ++b) {
-                if (b >= nb) break;
-                C *o = outb + (long)(b0 + b) * nd.rows + r;
-                atomicAdd(&o->x, ax[b]);
-                atomicAdd(&o->y, ay[b]);
+            for (int b = 0; b < NB; ++b) xs[threadIdx.x * NB + b] = acc.get(b);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < tl.nrow * NB; i += ST_THREADS) {
+            const int r = i / NB, b = i % NB;
+            if (b >= nb) continue;
+            C v = xs[i];
+            for (int q = 1; q < groups; ++q) v = v + xs[i + q * tl.nrow * NB];
+            C neg;
+            neg.x = -v.x;
+            neg.y = -v.y;
+            if (r < tl.nown) {
+                C *dst = Y + (long)(tl.out + r) * nrhs + b0 + b;
+                if (FWD) {
+                    if (tl.full) *dst = v;
+                    else add_to(dst, v);
+                } else {
+                    if (tl.full) *dst = __ldcg(dst) - v;
+                    else add_to(dst, neg);
+                }
+            } else {
+                add_to(W + (long)bnd[tl.bout + r - tl.nown] * nrhs + b0 + b, neg);
             }
         }
     }
+}
+
+// W[u][b] = b[b][c][point], Y = 0; and x[b][c][point] = Y[u][b]
+template <typename C>
+__global__ void k_nd_enter(C *W, C *Y, const C *__restrict__ in, const int *__restrict__ ptof, int D, long npts, int nrhs)
+{
+    const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long u = gid / nrhs, b = gid - u * nrhs;
+    pdl_wait_and_trigger();
+    if (u >= D * npts) return;
+    const int rank = (int)(u / D), c = (int)(u - (long)rank * D);
+    W[gid] = in[(b * D + c) * npts + ptof[rank]];
+    Y[gid] = czero<C>();
+}
+template <typename C>
+__global__ void k_nd_leave(C *out, const C *Y, const int *__restrict__ rankof, int D, long npts, int nrhs)
+{
+    const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long bc = gid / npts, pt = gid - bc * npts, b = bc / D, c = bc - b * D;
+    pdl_wait_and_trigger();
+    if (b >= nrhs) return;
+    out[gid] = __ldcg(Y + ((long)rankof[pt] * D + c) * nrhs + b);
 }
 
 // scale[c] = largest |component| of column c of an (m x ncol, ld m) block (1 if zero)
@@ -422,66 +504,6 @@ __global__ void k_to_half(__half2 *dst, const float2 *__restrict__ src, int m, i
     dst[gid] = __floats2half2_rn(v.x * inv, v.y * inv);
 }
 
-// node whose element range [unit[i] * nrhs, unit[i+1] * nrhs) holds gid
-__device__ __forceinline__ int find_node(const long *__restrict__ unit, int nn, long gid, int nrhs)
-{
-    int lo = 0, hi = nn - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) / 2;
-        if (unit[mid] * nrhs <= gid) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
-// packed input of every node of a level: own (which = 0) or boundary (1) unknowns of w
-template <typename C>
-__global__ void k_level_gather(C *packed, const C *__restrict__ w, const LevelNode *__restrict__ nodes,
-                               const long *__restrict__ in_units, const int *__restrict__ pts, int nn, long npts,
-                               int D, int nrhs, int which)
-{
-    long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= in_units[nn] * nrhs) return;
-    const int id = find_node(in_units, nn, gid, nrhs);
-    const LevelNode nd = nodes[id];
-    long e = gid - in_units[id] * nrhs;
-    long r = e % nd.cols, b = e / nd.cols;
-    int pt = pts[(which ? nd.bnd_pts : nd.own_pts) + (int)(r / D)];
-    packed[gid] = w[(b * D + (r % D)) * npts + pt];
-}
-
-// forward (mode 0): w_own = out[0:o3], w_bnd -= out[o3:] (siblings share
-// boundaries: atomic); backward (mode 1): w_own -= out
-template <typename C>
-__global__ void k_level_scatter(C *w, const C *__restrict__ packed, const LevelNode *__restrict__ nodes,
-                                const long *__restrict__ out_units, const int *__restrict__ pts, int nn, long npts,
-                                int D, int nrhs, int mode)
-{
-    long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= out_units[nn] * nrhs) return;
-    const int id = find_node(out_units, nn, gid, nrhs);
-    const LevelNode nd = nodes[id];
-    long e = gid - out_units[id] * nrhs;
-    long r = e % nd.rows, b = e / nd.rows;
-    C v = packed[gid];
-    const int o3 = D * nd.nown;
-    if (r < o3) {
-        long g = (b * D + (r % D)) * npts + pts[nd.own_pts + (int)(r / D)];
-        if (mode == 0) {
-            w[g] = v;
-        } else {
-            C u = w[g];
-            u.x -= v.x;
-            u.y -= v.y;
-            w[g] = u;
-        }
-    } else {
-        long rb = r - o3;
-        long g = (b * D + (rb % D)) * npts + pts[nd.bnd_pts + (int)(rb / D)];
-        atomicAdd(&w[g].x, -v.x);
-        atomicAdd(&w[g].y, -v.y);
-    }
-}
-
 } // namespace
 
 // ---------------------------------------------------------------- factor object
@@ -502,25 +524,20 @@ struct NDFactor {
     DevBuf front, stack, work, info; // factor scratch (released after factoring)
     DevBuf solve_ws;
     size_t max_front_unknowns = 0, max_own3 = 0, max_bnd3 = 0;
-    // level tables for the batched solve; levels[0] is the deepest
+    // tiles of the solve's levels; levels[0] is the deepest
     struct Level {
-        int nn_f, nn_b;                // nodes in the forward / backward tables
-        long nodes_f, nodes_b;         // offsets into the LevelNode table
-        long units_f_in, units_f_out, units_b_in, units_b_out; // offsets into the unit table (nn+1 each)
-        long tiles_f, tiles_b;         // offsets into the tile table
+        long tiles_f, tiles_b; // offsets into the tile table: forward (G), backward (X)
         int ntiles_f, ntiles_b;
-        long pack_f_in, pack_f_out, pack_b_in, pack_b_out; // packed sizes per RHS
     };
     std::vector<Level> levels;
-    DevBuf lv_nodes, lv_units, lv_tiles;
-    long max_pack_in = 0, max_pack_out = 0;
+    DevBuf st_tiles, st_bnd, st_rank, st_point; // tiles, boundary unknowns, rank of each point and back
     DenseWork *dense = nullptr; // Gauss-Jordan workspace
     ~NDFactor()
     {
         spm_dense_work_free(dense);
         pts.release(); maps.release(); rels.release(); fac.release(); piv.release();
         front.release(); stack.release(); work.release(); info.release(); solve_ws.release();
-        lv_nodes.release(); lv_units.release(); lv_tiles.release(); scales.release();
+        st_tiles.release(); st_bnd.release(); st_rank.release(); st_point.release(); scales.release();
     }
 };
 
@@ -578,6 +595,90 @@ int build_tree(std::vector<Node> &nodes, const int lo[3], const int hi[3], int v
 }
 
 } // namespace
+
+// Elimination ranks, boundary lists and tiles of every level.  A level's tiles hold
+// at most st_rows rows (a node's rows are cut evenly) and as many columns as leave
+// about eight tiles for every SM, between 8 and ST_COLS: levels of few nodes spread
+// over the chip, levels of many read long stretches and add each row's sum once.
+template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std::vector<int> &pts)
+{
+    using C = typename cplx_of<R>::type;
+    const std::vector<Node> &nodes = F->nodes;
+    const int NN = (int)nodes.size(), D = F->D;
+    std::vector<int> rank(F->npts), point(F->npts), bnd;
+    std::vector<int> base(NN), boff(NN);
+    int next = 0;
+    for (int id = 0; id < NN; ++id) {
+        base[id] = D * next;
+        for (int a = 0; a < nodes[id].nown; ++a, ++next) {
+            const int p = pts[nodes[id].own_off + a];
+            rank[p] = next;
+            point[next] = p;
+        }
+    }
+    int maxd = 0;
+    for (int id = 0; id < NN; ++id) {
+        const Node &nd = nodes[id];
+        boff[id] = (int)bnd.size();
+        for (int b = 0; b < nd.nbnd; ++b)
+            for (int c = 0; c < D; ++c) bnd.push_back(D * rank[pts[nd.bnd_off + b]] + c);
+        maxd = std::max(maxd, nd.depth);
+    }
+    std::vector<std::vector<int>> at(maxd + 1);
+    for (int id = 0; id < NN; ++id) at[nodes[id].depth].push_back(id);
+    std::vector<SolveTile> tt;
+    auto cut = [&](const std::vector<int> &ids, bool fwd, long &first, int &count) {
+        first = (long)tt.size();
+        double level = 0;
+        for (int id : ids) {
+            const double o = D * (double)nodes[id].nown, b = D * (double)nodes[id].nbnd;
+            level += fwd ? (o + b) * o : o * b;
+        }
+        const double per_tile = level / (8 * 152);
+        for (int id : ids) {
+            const Node &nd = nodes[id];
+            const int o = D * nd.nown, b = D * nd.nbnd;
+            const int rows = fwd ? o + b : o, cols = fwd ? o : b;
+            if (cols == 0) continue;
+            const int nr = (rows + st_rows<C>() - 1) / st_rows<C>(), rt = (rows + nr - 1) / nr;
+            int ct = (int)std::min<double>(ST_COLS, std::max(8.0, per_tile / rt));
+            const int nc = (cols + ct - 1) / ct;
+            ct = (cols + nc - 1) / nc;
+            for (int r0 = 0; r0 < rows; r0 += rt)
+                for (int c0 = 0; c0 < cols; c0 += ct) {
+                    SolveTile t;
+                    t.ld = rows;
+                    t.nrow = std::min(rt, rows - r0);
+                    t.ncol = std::min(ct, cols - c0);
+                    t.mat = nd.fac_off + (fwd ? 0 : (long)(o + b) * o) + (long)c0 * rows + r0;
+                    t.scale = nd.scale_off + (fwd ? 0 : o) + c0;
+                    t.in = fwd ? base[id] + c0 : boff[id] + c0;
+                    t.out = base[id] + r0;
+                    t.nown = std::max(0, std::min(t.nrow, o - r0));
+                    t.bout = boff[id] + std::max(0, r0 - o);
+                    t.full = t.ncol == cols;
+                    tt.push_back(t);
+                }
+        }
+        count = (int)((long)tt.size() - first);
+    };
+    F->levels.clear();
+    for (int d = maxd; d >= 0; --d) {
+        NDFactor::Level lv;
+        cut(at[d], true, lv.tiles_f, lv.ntiles_f);
+        cut(at[d], false, lv.tiles_b, lv.ntiles_b);
+        F->levels.push_back(lv);
+    }
+    auto put = [](DevBuf &buf, const void *src, size_t bytes) -> spm_status {
+        SPM_TRY(buf.ensure(std::max<size_t>(bytes, 1)));
+        if (bytes) SPM_CUDA_TRY(cudaMemcpy(buf.ptr, src, bytes, cudaMemcpyHostToDevice));
+        return SPM_OK;
+    };
+    SPM_TRY(put(F->st_tiles, tt.data(), sizeof(SolveTile) * tt.size()));
+    SPM_TRY(put(F->st_bnd, bnd.data(), sizeof(int) * bnd.size()));
+    SPM_TRY(put(F->st_rank, rank.data(), sizeof(int) * rank.size()));
+    return put(F->st_point, point.data(), sizeof(int) * point.size());
+}
 
 template <typename R>
 static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store, int variant)
@@ -963,134 +1064,58 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
         spm_set_error("a grid barrier of the Gauss-Jordan panel expired (code %d)", hinfo[0]);
         return SPM_ERR_TIMEOUT;
     }
-    // level tables for the batched solve
-    {
-        int maxd = 0;
-        for (const Node &nd : nodes) maxd = std::max(maxd, nd.depth);
-        std::vector<LevelNode> tn;
-        std::vector<long> tu;
-        std::vector<Tile> tt;
-        F->levels.clear();
-        F->max_pack_in = F->max_pack_out = 0;
-        auto add_table = [&](const std::vector<int> &ids, bool fwd, int &nn, long &nodes_off, long &uin, long &uout,
-                             long &tiles_off, int &ntiles, long &pin, long &pout) {
-            nodes_off = (long)tn.size();
-            tiles_off = (long)tt.size();
-            std::vector<long> ui(1, 0), uo(1, 0);
-            nn = 0;
-            for (int id : ids) {
-                const Node &nd = nodes[id];
-                const int o3 = D * nd.nown, b3 = D * nd.nbnd, f = o3 + b3;
-                LevelNode L;
-                L.rows = fwd ? f : o3;
-                L.cols = fwd ? o3 : b3;
-                if (L.cols == 0) continue;
-                L.mat_off = fwd ? nd.fac_off : nd.fac_off + (long)f * o3;
-                L.scale_off = fwd ? nd.scale_off : nd.scale_off + o3;
-                L.in_unit = ui.back();
-                L.out_unit = uo.back();
-                L.own_pts = (int)nd.own_off;
-                L.bnd_pts = (int)nd.bnd_off;
-                L.nown = nd.nown;
-                L.nbnd = nd.nbnd;
-                for (int r0 = 0; r0 < L.rows; r0 += GT_ROWS)
-                    for (int c0 = 0; c0 < L.cols; c0 += GT_COLS) tt.push_back(Tile{nn, r0, c0});
-                tn.push_back(L);
-                ui.push_back(ui.back() + L.cols);
-                uo.push_back(uo.back() + L.rows);
-                ++nn;
-            }
-            uin = (long)tu.size();
-            tu.insert(tu.end(), ui.begin(), ui.end());
-            uout = (long)tu.size();
-            tu.insert(tu.end(), uo.begin(), uo.end());
-            ntiles = (int)(tt.size() - tiles_off);
-            pin = ui.back();
-            pout = uo.back();
-            F->max_pack_in = std::max(F->max_pack_in, pin);
-            F->max_pack_out = std::max(F->max_pack_out, pout);
-        };
-        for (int d = maxd; d >= 0; --d) {
-            std::vector<int> ids;
-            for (int id = 0; id < NN; ++id) if (nodes[id].depth == d) ids.push_back(id);
-            NDFactor::Level lv;
-            add_table(ids, true, lv.nn_f, lv.nodes_f, lv.units_f_in, lv.units_f_out, lv.tiles_f, lv.ntiles_f,
-                      lv.pack_f_in, lv.pack_f_out);
-            add_table(ids, false, lv.nn_b, lv.nodes_b, lv.units_b_in, lv.units_b_out, lv.tiles_b, lv.ntiles_b,
-                      lv.pack_b_in, lv.pack_b_out);
-            F->levels.push_back(lv);
-        }
-        SPM_TRY(F->lv_nodes.ensure(sizeof(LevelNode) * tn.size()));
-        SPM_TRY(F->lv_units.ensure(sizeof(long) * tu.size()));
-        SPM_TRY(F->lv_tiles.ensure(sizeof(Tile) * std::max<size_t>(tt.size(), 1)));
-        SPM_CUDA_TRY(cudaMemcpy(F->lv_nodes.ptr, tn.data(), sizeof(LevelNode) * tn.size(), cudaMemcpyHostToDevice));
-        SPM_CUDA_TRY(cudaMemcpy(F->lv_units.ptr, tu.data(), sizeof(long) * tu.size(), cudaMemcpyHostToDevice));
-        if (!tt.empty())
-            SPM_CUDA_TRY(cudaMemcpy(F->lv_tiles.ptr, tt.data(), sizeof(Tile) * tt.size(), cudaMemcpyHostToDevice));
+    return build_solve_tiles<R>(F, pts);
+}
+
+template <typename C, typename S, int NB>
+static void launch_levels(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStream_t s)
+{
+    const float *scales = F->scales.as<float>();
+    const SolveTile *tiles = F->st_tiles.as<SolveTile>();
+    const int *bnd = F->st_bnd.as<int>(), NL = (int)F->levels.size();
+    for (int l = 0; l < NL; ++l) { // forward, deepest level first
+        const NDFactor::Level &lv = F->levels[l];
+        if (lv.ntiles_f > 0)
+            launch_pdl(k_nd_level<C, S, NB, true>, dim3(lv.ntiles_f), dim3(ST_THREADS), 0, s, M, scales, tiles + lv.tiles_f,
+                       bnd, W, Y, nrhs);
     }
-    return SPM_OK;
+    for (int l = NL - 1; l >= 0; --l) { // backward, root first
+        const NDFactor::Level &lv = F->levels[l];
+        if (lv.ntiles_b > 0)
+            launch_pdl(k_nd_level<C, S, NB, false>, dim3(lv.ntiles_b), dim3(ST_THREADS), 0, s, M, scales, tiles + lv.tiles_b,
+                       bnd, W, Y, nrhs);
+    }
+}
+
+// right-hand sides per pass over a tile: a tile is read once per group of NB
+template <typename C, typename S>
+static void launch_solve(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStream_t s)
+{
+    if (nrhs == 1) launch_levels<C, S, 1>(F, M, W, Y, nrhs, s);
+    else if (nrhs == 2) launch_levels<C, S, 2>(F, M, W, Y, nrhs, s);
+    else if (nrhs <= 4) launch_levels<C, S, 4>(F, M, W, Y, nrhs, s);
+    else if (nrhs <= 8 || sizeof(C) == 16) launch_levels<C, S, 8>(F, M, W, Y, nrhs, s);
+    else launch_levels<C, S, sizeof(C) == 16 ? 8 : 16>(F, M, W, Y, nrhs, s);
 }
 
 template <typename R>
 static spm_status solve_typed(NDFactor *F, const void *bv, void *xv, int nrhs, cudaStream_t s)
 {
     using C = typename cplx_of<R>::type;
-    const long npts = F->npts;
-    const int D = F->D;
-    C *x = reinterpret_cast<C *>(xv);
-    SPM_CUDA_TRY(cudaMemcpyAsync(x, bv, sizeof(C) * D * npts * nrhs, cudaMemcpyDeviceToDevice, s));
-    const size_t pin = (size_t)F->max_pack_in * nrhs, pout = (size_t)F->max_pack_out * nrhs;
-    SPM_TRY(F->solve_ws.ensure(sizeof(C) * (pin + pout)));
-    C *in = F->solve_ws.as<C>();
-    C *out = in + pin;
-    const int *dpts = F->pts.as<int>();
-    const C *fac = F->fac.as<C>();
-    const __half2 *fac16 = F->fac.as<__half2>();
-    const float *scales = F->scales.as<float>();
-    const LevelNode *tn = F->lv_nodes.as<LevelNode>();
-    // right-hand sides per pass over a factor tile: the tile is read once per
-    // group, so blocks of many RHS read the factor nrhs / GT_NB times
-    auto gemv = [&](int ntiles, const LevelNode *nodes, const Tile *tiles) {
-        if constexpr (sizeof(R) == 4) {
-            if (F->half_store) {
-                if (nrhs == 1) k_level_gemv<C, 1, __half2><<<ntiles, GT_ROWS, 0, s>>>(fac16, scales, nodes, tiles, in, out, nrhs);
-                else if (nrhs < 8) k_level_gemv<C, 4, __half2><<<ntiles, GT_ROWS, 0, s>>>(fac16, scales, nodes, tiles, in, out, nrhs);
-                else if (nrhs < 16) k_level_gemv<C, 8, __half2><<<ntiles, GT_ROWS, 0, s>>>(fac16, scales, nodes, tiles, in, out, nrhs);
-                else k_level_gemv<C, 16, __half2><<<ntiles, GT_ROWS, 0, s>>>(fac16, scales, nodes, tiles, in, out, nrhs);
-                return;
-            }
-            if (nrhs >= 16) {
-                k_level_gemv<C, 16, C><<<ntiles, GT_ROWS, 0, s>>>(fac, scales, nodes, tiles, in, out, nrhs);
-                return;
-            }
-        }
-        if (nrhs == 1) k_level_gemv<C, 1, C><<<ntiles, GT_ROWS, 0, s>>>(fac, scales, nodes, tiles, in, out, nrhs);
-        else if (nrhs < 8) k_level_gemv<C, 4, C><<<ntiles, GT_ROWS, 0, s>>>(fac, scales, nodes, tiles, in, out, nrhs);
-        else k_level_gemv<C, 8, C><<<ntiles, GT_ROWS, 0, s>>>(fac, scales, nodes, tiles, in, out, nrhs);
-    };
-    const long *tu = F->lv_units.as<long>();
-    const Tile *tt = F->lv_tiles.as<Tile>();
-    const int NL = (int)F->levels.size();
-    for (int l = 0; l < NL; ++l) { // forward, deepest level first
-        const NDFactor::Level &lv = F->levels[l];
-        if (lv.nn_f == 0) continue;
-        k_level_gather<C><<<blocks(lv.pack_f_in * nrhs), 256, 0, s>>>(in, x, tn + lv.nodes_f, tu + lv.units_f_in, dpts,
-                                                                       lv.nn_f, npts, D, nrhs, 0);
-        SPM_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(C) * lv.pack_f_out * nrhs, s));
-        gemv(lv.ntiles_f, tn + lv.nodes_f, tt + lv.tiles_f);
-        k_level_scatter<C><<<blocks(lv.pack_f_out * nrhs), 256, 0, s>>>(x, out, tn + lv.nodes_f, tu + lv.units_f_out,
-                                                                         dpts, lv.nn_f, npts, D, nrhs, 0);
+    const long N = F->D * F->npts;
+    SPM_TRY(F->solve_ws.ensure(sizeof(C) * 2 * N * nrhs));
+    C *W = F->solve_ws.as<C>(), *Y = W + N * nrhs;
+    const unsigned grid = blocks(N * nrhs);
+    launch_pdl(k_nd_enter<C>, dim3(grid), dim3(256), 0, s, W, Y, reinterpret_cast<const C *>(bv),
+               F->st_point.as<const int>(), F->D, F->npts, nrhs);
+    bool half = false;
+    if constexpr (sizeof(R) == 4) {
+        half = F->half_store;
+        if (half) launch_solve<C, __half2>(F, F->fac.as<__half2>(), W, Y, nrhs, s);
     }
-    for (int l = NL - 1; l >= 0; --l) { // backward, root first
-        const NDFactor::Level &lv = F->levels[l];
-        if (lv.nn_b == 0) continue;
-        k_level_gather<C><<<blocks(lv.pack_b_in * nrhs), 256, 0, s>>>(in, x, tn + lv.nodes_b, tu + lv.units_b_in, dpts,
-                                                                       lv.nn_b, npts, D, nrhs, 1);
-        SPM_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(C) * lv.pack_b_out * nrhs, s));
-        gemv(lv.ntiles_b, tn + lv.nodes_b, tt + lv.tiles_b);
-        k_level_scatter<C><<<blocks(lv.pack_b_out * nrhs), 256, 0, s>>>(x, out, tn + lv.nodes_b, tu + lv.units_b_out,
-                                                                         dpts, lv.nn_b, npts, D, nrhs, 1);
-    }
+    if (!half) launch_solve<C, C>(F, F->fac.as<C>(), W, Y, nrhs, s);
+    launch_pdl(k_nd_leave<C>, dim3(grid), dim3(256), 0, s, reinterpret_cast<C *>(xv), (const C *)Y,
+               F->st_rank.as<const int>(), F->D, F->npts, nrhs);
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
 }
