@@ -1340,7 +1340,7 @@ spm_status apply_A_typed(spm_problem_s *P, const void *xv, void *yv, int nrhs, c
     return SPM_OK;
 }
 
-// Q gather in one launch of 256-thread blocks of three kinds (block-uniform
+// Q gather in complex64, one launch of 128-thread blocks of three kinds (block-uniform
 // branch), boundary blocks first so that their latency overlaps the interior:
 // * face blocks: the points with exactly one coordinate on the boundary belong
 //   to one of six face classes; a block owns a 32 x 4 tile of one face, stages
@@ -1367,16 +1367,13 @@ constexpr int QF_HU = QF_U + 2, QF_HW = QF_W + 2, QF_HALO = 3 * 2 * QF_HW * QF_H
 constexpr int Q_SMEM = (3 * QH > QF_HALO + 162) ? 3 * QH : QF_HALO + 162; // complex elements
 static_assert(QX * QY == Q_THREADS && QF_U * QF_W == Q_THREADS, "Q block shapes");
 
-template <typename C> struct QInterior {
-    C a[243]; // [d][o][c], o = (o3+1)*9 + (o2+1)*3 + (o1+1)
-};
-// complex64: each coefficient a as the packed pairs (a.x, a.x, -a.y, a.y), so a
-// complex MAC acc += a v is two packed FP32x2 FMAs, (a.x, a.x) (v.x, v.y) and
-// (-a.y, a.y) (v.y, v.x)
-template <> struct QInterior<float2> {
+// interior coefficients [d][o][c], o = (o3+1)*9 + (o2+1)*3 + (o1+1): each coefficient a
+// as the packed pairs (a.x, a.x, -a.y, a.y), so a complex MAC acc += a v is two packed
+// FP32x2 FMAs, (a.x, a.x) (v.x, v.y) and (-a.y, a.y) (v.y, v.x)
+struct QInterior {
     float4 a[243];
 };
-static_assert(sizeof(QInterior<float2>) + 64 <= 4096, "kernel parameter space");
+static_assert(sizeof(QInterior) + 64 <= 4096, "kernel parameter space");
 
 // edge point number e (0 <= e < 12 (n-2) + 8) -> (i1, i2, i3): corners, then the
 // edges along x, y, z (four each)
@@ -1395,9 +1392,8 @@ __device__ __forceinline__ void edge_point(int e, int n, int &i1, int &i2, int &
     else { i1 = b0; i2 = b1; i3 = t; }
 }
 
-template <typename C>
-__device__ __forceinline__ void q_interior_block(int blk, const C *__restrict__ vb, const QInterior<C> &qa,
-                                                 C *__restrict__ yb, int n, C *sv)
+__device__ __forceinline__ void q_interior_block(int blk, const float2 *__restrict__ vb, const QInterior &qa,
+                                                 float2 *__restrict__ yb, int n, float2 *sv)
 {
     const long n3 = (long)n * n * n;
     const int m = n - 2; // interior extent
@@ -1412,7 +1408,7 @@ __device__ __forceinline__ void q_interior_block(int blk, const C *__restrict__ 
         int hx = h % QHX, hy = (h / QHX) % QHY, hz = h / (QHX * QHY);
         int gx = tx0 + hx - 1, gy = ty0 + hy - 1, gz = tz0 + hz - 1;
         const bool in = gx < n && gy < n && gz < n;
-        cp_async_zfill<sizeof(C)>(&sv[i], in ? vb + d * n3 + ((long)gz * n + gy) * n + gx : vb, in);
+        cp_async_zfill<sizeof(float2)>(&sv[i], in ? vb + d * n3 + ((long)gz * n + gy) * n + gx : vb, in);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -1420,9 +1416,9 @@ __device__ __forceinline__ void q_interior_block(int blk, const C *__restrict__ 
     const int lx = threadIdx.x % QX, ly = threadIdx.x / QX;
     const int i1 = tx0 + lx, i2 = ty0 + ly;
     if (i1 > n - 2 || i2 > n - 2) return;
-    C acc[QZ][3];
+    float2 acc[QZ][3];
 #pragma unroll
-    for (int q = 0; q < QZ; ++q) acc[q][0] = acc[q][1] = acc[q][2] = czero<C>();
+    for (int q = 0; q < QZ; ++q) acc[q][0] = acc[q][1] = acc[q][2] = czero<float2>();
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
@@ -1430,35 +1426,22 @@ __device__ __forceinline__ void q_interior_block(int blk, const C *__restrict__ 
 #pragma unroll
             for (int o1 = -1; o1 <= 1; ++o1) {
                 // the z-column (d, i2 + o2, i1 + o1) over the tile's QZ + 2 halo planes
-                C col[QZ + 2];
+                float2 col[QZ + 2];
 #pragma unroll
                 for (int j = 0; j < QZ + 2; ++j) col[j] = sv[d * QH + (j * QHY + ly + 1 + o2) * QHX + lx + 1 + o1];
-                if constexpr (std::is_same<C, float2>::value) {
-                    float2 cs[QZ + 2]; // (im, re) of each value, for the second packed FMA
+                float2 cs[QZ + 2]; // (im, re) of each value, for the second packed FMA
 #pragma unroll
-                    for (int j = 0; j < QZ + 2; ++j) cs[j] = make_float2(col[j].y, col[j].x);
+                for (int j = 0; j < QZ + 2; ++j) cs[j] = make_float2(col[j].y, col[j].x);
 #pragma unroll
-                    for (int o3 = -1; o3 <= 1; ++o3) {
-                        const int o = (o3 + 1) * 9 + (o2 + 1) * 3 + (o1 + 1);
+                for (int o3 = -1; o3 <= 1; ++o3) {
+                    const int o = (o3 + 1) * 9 + (o2 + 1) * 3 + (o1 + 1);
 #pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            const float4 a = qa.a[(d * 27 + o) * 3 + c];
-                            const float2 ar = make_float2(a.x, a.y), ai = make_float2(a.z, a.w);
+                    for (int c = 0; c < 3; ++c) {
+                        const float4 a = qa.a[(d * 27 + o) * 3 + c];
+                        const float2 ar = make_float2(a.x, a.y), ai = make_float2(a.z, a.w);
 #pragma unroll
-                            for (int q = 0; q < QZ; ++q)
-                                acc[q][c] = __ffma2_rn(ai, cs[q + o3 + 1], __ffma2_rn(ar, col[q + o3 + 1], acc[q][c]));
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int o3 = -1; o3 <= 1; ++o3) {
-                        const int o = (o3 + 1) * 9 + (o2 + 1) * 3 + (o1 + 1);
-#pragma unroll
-                        for (int c = 0; c < 3; ++c) {
-                            const C a = qa.a[(d * 27 + o) * 3 + c];
-#pragma unroll
-                            for (int q = 0; q < QZ; ++q) acc[q][c] = cfma(a, col[q + o3 + 1], acc[q][c]);
-                        }
+                        for (int q = 0; q < QZ; ++q)
+                            acc[q][c] = __ffma2_rn(ai, cs[q + o3 + 1], __ffma2_rn(ar, col[q + o3 + 1], acc[q][c]));
                     }
                 }
             }
@@ -1473,11 +1456,10 @@ __device__ __forceinline__ void q_interior_block(int blk, const C *__restrict__ 
     }
 }
 
-template <typename C>
-__device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, const C *__restrict__ qtab,
-                                             C *__restrict__ yb, int n, C *sv)
+__device__ __forceinline__ void q_face_block(int blk, const float2 *__restrict__ vb, const float2 *__restrict__ qtab,
+                                             float2 *__restrict__ yb, int n, float2 *sv)
 {
-    C *sa = sv + QF_HALO; // 162 coefficients [d][la][ou][ow][c]
+    float2 *sa = sv + QF_HALO; // 162 coefficients [d][la][ou][ow][c]
     const long n3 = (long)n * n * n, n2 = (long)n * n;
     const int m = n - 2;
     const int tiles_u = (m + QF_U - 1) / QF_U, tiles_w = (m + QF_W - 1) / QF_W;
@@ -1492,7 +1474,7 @@ __device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, 
     const int ia0 = side ? n - 1 : 0;
     const int cf = side ? 2 : 0;
     const int cls = (a == 0 ? cf : 1) + 3 * (a == 1 ? cf : 1) + 9 * (a == 2 ? cf : 1);
-    const C *al = qtab + (long)cls * 243;
+    const float2 *al = qtab + (long)cls * 243;
     for (int i = threadIdx.x; i < 162; i += Q_THREADS) {
         const int c = i % 3, l = (i / 3) % 18, d = i / 54;
         const int la = l / 9, ou = (l / 3) % 3 - 1, ow = l % 3 - 1;
@@ -1507,7 +1489,7 @@ __device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, 
         const int hu = i % QF_HU, hw = (i / QF_HU) % QF_HW, la = (i / (QF_HU * QF_HW)) % 2, d = i / (2 * QF_HU * QF_HW);
         const int gu = u0 + hu, gw = w0 + hw; // halo starts one point before the first face point (u = 1)
         const bool in = gu < n && gw < n;
-        cp_async_zfill<sizeof(C)>(&sv[i], in ? vb + d * n3 + (ia0 + (la ? inward : 0)) * sa_ + gu * su + gw * sw : vb, in);
+        cp_async_zfill<sizeof(float2)>(&sv[i], in ? vb + d * n3 + (ia0 + (la ? inward : 0)) * sa_ + gu * su + gw * sw : vb, in);
     }
     cp_async_commit();
     cp_async_wait<0>();
@@ -1515,7 +1497,7 @@ __device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, 
     const int lu = threadIdx.x % QF_U, lw = threadIdx.x / QF_U;
     const int pu = 1 + u0 + lu, pw = 1 + w0 + lw;
     if (pu > m || pw > m) return;
-    C acc0 = czero<C>(), acc1 = czero<C>(), acc2 = czero<C>();
+    float2 acc0 = czero<float2>(), acc1 = czero<float2>(), acc2 = czero<float2>();
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
@@ -1524,8 +1506,8 @@ __device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, 
             for (int ou = -1; ou <= 1; ++ou)
 #pragma unroll
                 for (int ow = -1; ow <= 1; ++ow) {
-                    const C val = sv[((d * 2 + la) * QF_HW + (lw + 1 + ow)) * QF_HU + (lu + 1 + ou)];
-                    const C *ar = sa + ((d * 18 + la * 9 + (ou + 1) * 3 + (ow + 1)) * 3);
+                    const float2 val = sv[((d * 2 + la) * QF_HW + (lw + 1 + ow)) * QF_HU + (lu + 1 + ou)];
+                    const float2 *ar = sa + ((d * 18 + la * 9 + (ou + 1) * 3 + (ow + 1)) * 3);
                     acc0 = cfma(ar[0], val, acc0);
                     acc1 = cfma(ar[1], val, acc1);
                     acc2 = cfma(ar[2], val, acc2);
@@ -1536,9 +1518,8 @@ __device__ __forceinline__ void q_face_block(int blk, const C *__restrict__ vb, 
     yb[2 * n3 + i] = acc2;
 }
 
-template <typename C>
-__device__ __forceinline__ void q_edge_block(int blk, const C *__restrict__ vb, const C *__restrict__ qtab,
-                                             C *__restrict__ yb, int n, int nedge)
+__device__ __forceinline__ void q_edge_block(int blk, const float2 *__restrict__ vb, const float2 *__restrict__ qtab,
+                                             float2 *__restrict__ yb, int n, int nedge)
 {
     const long n3 = (long)n * n * n;
     const int e = blk * (Q_THREADS / 32) + (int)(threadIdx.x >> 5);
@@ -1549,8 +1530,8 @@ __device__ __forceinline__ void q_edge_block(int blk, const C *__restrict__ vb, 
     const int c1 = i1 == 0 ? 0 : (i1 == n - 1 ? 2 : 1);
     const int c2 = i2 == 0 ? 0 : (i2 == n - 1 ? 2 : 1);
     const int c3 = i3 == 0 ? 0 : (i3 == n - 1 ? 2 : 1);
-    const C *al = qtab + (long)(c1 + 3 * c2 + 9 * c3) * 243;
-    C acc0 = czero<C>(), acc1 = czero<C>(), acc2 = czero<C>();
+    const float2 *al = qtab + (long)(c1 + 3 * c2 + 9 * c3) * 243;
+    float2 acc0 = czero<float2>(), acc1 = czero<float2>(), acc2 = czero<float2>();
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         const int term = lane + 32 * k;
@@ -1558,8 +1539,8 @@ __device__ __forceinline__ void q_edge_block(int blk, const C *__restrict__ vb, 
         const int d = term / 27, o = term % 27;
         const int j1 = i1 + o % 3 - 1, j2 = i2 + (o / 3) % 3 - 1, j3 = i3 + o / 9 - 1;
         if (j1 < 0 || j2 < 0 || j3 < 0 || j1 >= n || j2 >= n || j3 >= n) continue;
-        const C val = vb[d * n3 + ((long)j3 * n + j2) * n + j1];
-        const C *ar = al + (d * 27 + o) * 3;
+        const float2 val = vb[d * n3 + ((long)j3 * n + j2) * n + j1];
+        const float2 *ar = al + (d * 27 + o) * 3;
         acc0 = cfma(ar[0], val, acc0);
         acc1 = cfma(ar[1], val, acc1);
         acc2 = cfma(ar[2], val, acc2);
@@ -1581,25 +1562,63 @@ __device__ __forceinline__ void q_edge_block(int blk, const C *__restrict__ vb, 
     }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(Q_THREADS) k_q(const typename cplx_of<R>::type *__restrict__ v,
-                                                 const QInterior<typename cplx_of<R>::type> qa,
-                                                 const typename cplx_of<R>::type *__restrict__ qtab,
-                                                 typename cplx_of<R>::type *__restrict__ y, int n, int face_blocks,
+__global__ void __launch_bounds__(Q_THREADS) k_q(const float2 *__restrict__ v,
+                                                 const QInterior qa,
+                                                 const float2 *__restrict__ qtab,
+                                                 float2 *__restrict__ y, int n, int face_blocks,
                                                  int edge_blocks, int nedge)
 {
     pdl_wait_and_trigger();
-    using C = typename cplx_of<R>::type;
     extern __shared__ unsigned char smem_raw[];
-    C *sv = reinterpret_cast<C *>(smem_raw); // Q_SMEM complex elements
+    float2 *sv = reinterpret_cast<float2 *>(smem_raw); // Q_SMEM complex elements
     const long n3 = (long)n * n * n;
     const long b = blockIdx.y;
-    const C *vb = v + b * 3 * n3;
-    C *yb = y + b * 3 * n3;
+    const float2 *vb = v + b * 3 * n3;
+    float2 *yb = y + b * 3 * n3;
     const int blk = blockIdx.x;
-    if (blk < face_blocks) q_face_block<C>(blk, vb, qtab, yb, n, sv);
-    else if (blk < face_blocks + edge_blocks) q_edge_block<C>(blk - face_blocks, vb, qtab, yb, n, nedge);
-    else q_interior_block<C>(blk - face_blocks - edge_blocks, vb, qa, yb, n, sv);
+    if (blk < face_blocks) q_face_block(blk, vb, qtab, yb, n, sv);
+    else if (blk < face_blocks + edge_blocks) q_edge_block(blk - face_blocks, vb, qtab, yb, n, nedge);
+    else q_interior_block(blk - face_blocks - edge_blocks, vb, qa, yb, n, sv);
+}
+
+// Q in complex128: one thread per (point, output component), values and coefficients
+// straight from the caches.  Bound: the FP64 pipe (two lanes per SM, so a warp's FMA
+// takes 16 cycles): 972 n^3 FMAs, 6.3 us at n = 16 and 1.37 ms at n = 96.  Loads are
+// nearly free beside that, and what counts is that every SM gets the same share of full
+// warps: the 32 x 4 x 4 tiles of the complex64 kernel left one tile's work on each of 16
+// SMs at n = 16 (157 us; this kernel 17 us) and half-empty tiles elsewhere (n = 64: 600
+// against 421 us, n = 96: 1780 against 1395 us).  In complex64 the tiles win from n = 16
+// on (n = 64: 21 against 33 us) and the two are equal below.
+template <typename C>
+__global__ void __launch_bounds__(Q_THREADS) k_q_direct(const C *__restrict__ v, const C *__restrict__ qtab,
+                                                        C *__restrict__ y, int n)
+{
+    pdl_wait_and_trigger();
+    const int n2 = n * n, n3 = n2 * n;
+    const int i = blockIdx.x * Q_THREADS + threadIdx.x, c = blockIdx.y;
+    if (i >= n3) return;
+    const int i1 = i % n, i2 = (i / n) % n, i3 = i / n2;
+    const bool lo[3] = {i1 > 0, i2 > 0, i3 > 0}, hi[3] = {i1 < n - 1, i2 < n - 1, i3 < n - 1};
+    const int cls = (lo[0] ? (hi[0] ? 1 : 2) : 0) + 3 * (lo[1] ? (hi[1] ? 1 : 2) : 0) + 9 * (lo[2] ? (hi[2] ? 1 : 2) : 0);
+    const C *al = qtab + cls * 243 + c;
+    const C *vb = v + (long)blockIdx.z * 3 * n3 + i;
+    C acc = czero<C>();
+#pragma unroll 1
+    for (int d = 0; d < 3; ++d, vb += n3, al += 81) {
+        C a[27], u[27]; // all loads of a component before its FMAs
+#pragma unroll
+        for (int o = 0; o < 27; ++o) {
+            const int o1 = o % 3 - 1, o2 = (o / 3) % 3 - 1, o3 = o / 9 - 1;
+            const bool in = (o1 == 0 || (o1 < 0 ? lo[0] : hi[0])) && (o2 == 0 || (o2 < 0 ? lo[1] : hi[1])) &&
+                            (o3 == 0 || (o3 < 0 ? lo[2] : hi[2]));
+            a[o] = al[3 * o];
+            u[o] = czero<C>();
+            if (in) u[o] = vb[o3 * n2 + o2 * n + o1];
+        }
+#pragma unroll
+        for (int o = 0; o < 27; ++o) acc = cfma(a[o], u[o], acc);
+    }
+    y[((long)blockIdx.z * 3 + c) * n3 + i] = acc;
 }
 
 template <typename R>
@@ -1608,12 +1627,19 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
     using C = typename cplx_of<R>::type;
     const int n = P->n;
     const C *qtab = sizeof(R) == 8 ? P->qtab128.as<C>() : P->qtab64.as<C>();
+    if constexpr (sizeof(R) == 8) {
+        const dim3 grid((unsigned)((n * n * n + Q_THREADS - 1) / Q_THREADS), 3, (unsigned)nrhs);
+        static const EvenPlacement even(k_q_direct<C>, Q_THREADS);
+        launch_pdl(k_q_direct<C>, grid, dim3(Q_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, (const C *)vv,
+                   qtab, (C *)yv, n);
+        SPM_CUDA_TRY(cudaGetLastError());
+        return SPM_OK;
+    } else {
     // interior coefficients (class 13) by value, from the host copy of the table
-    QInterior<C> qa;
+    QInterior qa;
     for (int i = 0; i < 243; ++i) {
-        const R ax = (R)P->qtab_h[2 * (13 * 243 + i)], ay = (R)P->qtab_h[2 * (13 * 243 + i) + 1];
-        if constexpr (sizeof(R) == 4) qa.a[i] = make_float4(ax, ax, -ay, ay);
-        else { qa.a[i].x = ax; qa.a[i].y = ay; }
+        const float ax = (float)P->qtab_h[2 * (13 * 243 + i)], ay = (float)P->qtab_h[2 * (13 * 243 + i) + 1];
+        qa.a[i] = make_float4(ax, ax, -ay, ay);
     }
     const C *v = reinterpret_cast<const C *>(vv);
     C *y = reinterpret_cast<C *>(yv);
@@ -1625,13 +1651,14 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
     constexpr size_t smem = sizeof(C) * Q_SMEM;
     static bool attr = false;
     if (!attr) {
-        allow_smem(k_q<R>, smem);
+        allow_smem(k_q, smem);
         attr = true;
     }
-    launch_pdl(k_q<R>, dim3((unsigned)(face_blocks + edge_blocks + interior_blocks), (unsigned)nrhs), dim3(Q_THREADS),
+    launch_pdl(k_q, dim3((unsigned)(face_blocks + edge_blocks + interior_blocks), (unsigned)nrhs), dim3(Q_THREADS),
                smem, s, v, qa, qtab, y, n, face_blocks, edge_blocks, nedge);
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
+    }
 }
 
 } // namespace

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -129,6 +130,38 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+
+// Even placement.  A grid that fits the chip at once may be placed unevenly (some SMs
+// full, others idle), which an FP64-bound kernel pays in full: 768 equal blocks of
+// k_q_direct on 152 SMs took 102 us, held to six on an SM 63 us.  smem_for(blocks) is
+// the dynamic shared memory with which at most ceil(blocks / SMs) blocks fit on an SM;
+// zero when the grid takes several waves, whose blocks go where there is room.  Made
+// once per kernel (the queries take microseconds).
+struct EvenPlacement {
+    int sms = 0, room = 0, most = 0, fixed = 0, per = 0;
+    template <typename K> EvenPlacement(K kernel, int threads)
+    {
+        int dev = 0;
+        cudaFuncAttributes fa = {};
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&room, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess)
+            per = 0;
+        fixed = 1024 + (int)fa.sharedSizeBytes; // reserved by the system, declared by the kernel
+        if (per > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            most - (int)fa.sharedSizeBytes) != cudaSuccess)
+            per = 0;
+    }
+    size_t smem_for(long blocks) const
+    {
+        if (per == 0) return 0;
+        const long want = (blocks + sms - 1) / sms;
+        if (want >= per) return 0;
+        return (size_t)std::max(0L, std::min<long>(room / (want + 1) + 1, most + 1024) - fixed); // one more would not fit
+    }
+};
 
 // ------------------------------------------------------------ device buffer
 // Owned device allocation: freed by release() or when the owner goes out of

@@ -459,29 +459,37 @@ __device__ __forceinline__ int cls_of(int i1, int i2, int n)
     return c1 + 3 * c2;
 }
 
-// (Q v)_{i,c} = sum_{s,d} qtab[cls][c][s][d] v^d_{i+o_s}
+// (Q v)_{i,c} = sum_{s,d} qtab[cls][c][s][d] v^d_{i+o_s}: one thread per (point, c), all
+// loads before the FMAs.  Complex128 is bound by the FP64 pipe (144 n^2 FMAs: 13 us at
+// n = 239), so blocks are small and evenly placed.
+constexpr int Q2_THREADS = 64;
 template <typename C>
-__global__ void k2_applyQ(const C *__restrict__ qtab, const C *__restrict__ v, C *__restrict__ y, int n, long total)
+__global__ void __launch_bounds__(Q2_THREADS) k2_applyQ(const C *__restrict__ qtab, const C *__restrict__ v,
+                                                        C *__restrict__ y, int n)
 {
-    const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= total) return;
-    const long N = (long)n * n, b = gid / N, i = gid - b * N;
+    pdl_wait_and_trigger();
+    const long N = (long)n * n, i = (long)blockIdx.x * Q2_THREADS + threadIdx.x;
+    const int c = blockIdx.y;
+    const long b = blockIdx.z;
+    if (i >= N) return;
     const int i1 = (int)(i % n), i2 = (int)(i / n);
-    const int cls = cls_of(i1, i2, n);
-    const C *vb = v + b * 2 * N;
-    C acc[2] = {czero<C>(), czero<C>()};
+    const C *q = qtab + (cls_of(i1, i2, n) * 2 + c) * 18, *vb = v + b * 2 * N + i;
+    C a[18], u[18];
+#pragma unroll
     for (int s = 0; s < 9; ++s) {
-        const int j1 = i1 + s % 3 - 1, j2 = i2 + s / 3 - 1;
-        if (j1 < 0 || j2 < 0 || j1 >= n || j2 >= n) continue;
-        const long j = (long)j2 * n + j1;
-        const C v0 = vb[j], v1 = vb[N + j];
-        for (int c = 0; c < 2; ++c) {
-            const C *q = qtab + ((cls * 2 + c) * 9 + s) * 2;
-            acc[c] = cfma(q[0], v0, cfma(q[1], v1, acc[c]));
+        const int o1 = s % 3 - 1, o2 = s / 3 - 1;
+        const bool in = i1 + o1 >= 0 && i1 + o1 < n && i2 + o2 >= 0 && i2 + o2 < n;
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+            a[2 * s + d] = q[2 * s + d];
+            u[2 * s + d] = czero<C>();
+            if (in) u[2 * s + d] = vb[d * N + (long)o2 * n + o1];
         }
     }
-    y[b * 2 * N + i] = acc[0];
-    y[b * 2 * N + N + i] = acc[1];
+    C acc = czero<C>();
+#pragma unroll
+    for (int s = 0; s < 18; ++s) acc = cfma(a[s], u[s], acc);
+    y[(b * 2 + c) * N + i] = acc;
 }
 
 // S[i][s][c][f] = alpha[(f,o),c] + beta[(f,o),c] m_j + beta[(2,o),c] p^f_j, j = i + o_s
@@ -739,13 +747,19 @@ spm_status spm2_apply_A_impl(spm2_problem_s *P, int prec, const void *x, void *y
     return prec == SPM_C128 ? apply_typed<double>(P, x, y, nrhs, s) : apply_typed<float>(P, x, y, nrhs, s);
 }
 
+template <typename C>
+static void launch_Q2(const C *qtab, const void *v, void *y, int n, int nrhs, cudaStream_t s)
+{
+    static const EvenPlacement even(k2_applyQ<C>, Q2_THREADS);
+    const dim3 grid(nb((long)n * n, Q2_THREADS), 2, (unsigned)nrhs);
+    launch_pdl(k2_applyQ<C>, grid, dim3(Q2_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, qtab,
+               reinterpret_cast<const C *>(v), reinterpret_cast<C *>(y), n);
+}
+
 spm_status spm2_apply_Q_impl(spm2_problem_s *P, int prec, const void *v, void *y, int nrhs, cudaStream_t s)
 {
-    const long total = (long)nrhs * P->n * P->n;
-    if (prec == SPM_C128)
-        k2_applyQ<double2><<<nb(total), 256, 0, s>>>(P->qtab128.as<double2>(), (const double2 *)v, (double2 *)y, P->n, total);
-    else
-        k2_applyQ<float2><<<nb(total), 256, 0, s>>>(P->qtab64.as<float2>(), (const float2 *)v, (float2 *)y, P->n, total);
+    if (prec == SPM_C128) launch_Q2<double2>(P->qtab128.as<double2>(), v, y, P->n, nrhs, s);
+    else launch_Q2<float2>(P->qtab64.as<float2>(), v, y, P->n, nrhs, s);
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
 }
