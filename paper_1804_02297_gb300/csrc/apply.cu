@@ -112,11 +112,11 @@ __global__ void __launch_bounds__(256) k2_xfwd(const typename cplx_of<R>::type *
     pdl_wait_and_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int E = line_elems(L), H = E / 2;
-    constexpr int T = L / E, n = L / 2, LPB = 256 / T > 0 ? 256 / T : 1, LS = L + L / 8;
+    constexpr int T = L / E, n = L / 2, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
     C *sm = reinterpret_cast<C *>(smem_raw);
     const int line = threadIdx.x / T, t = threadIdx.x % T;
-    const int g = blockIdx.x * LPB + line;
+    const int g = blockIdx.x * (blockDim.x / T) + line;
     const bool ok = g < nrows;
     const long n2 = (long)n * n, n3 = n2 * n;
     const long b = ok ? g / n2 : 0, zy = ok ? g - b * n2 : 0;
@@ -788,11 +788,11 @@ __global__ void __launch_bounds__(256) k2_xinv(const typename cplx_of<R>::type *
     pdl_wait_and_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int E = line_elems(L), H = E / 2;
-    constexpr int T = L / E, n = L / 2, LPB = 256 / T > 0 ? 256 / T : 1, LS = L + L / 8;
+    constexpr int T = L / E, n = L / 2, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
     C *sm = reinterpret_cast<C *>(smem_raw);
     const int line = threadIdx.x / T, t = threadIdx.x % T;
-    const long g = (long)blockIdx.x * LPB + line;
+    const long g = (long)blockIdx.x * (blockDim.x / T) + line;
     const bool ok = g < nrows;
     C v[E];
 #pragma unroll
@@ -1058,6 +1058,14 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     constexpr int n = L / 2, T = L / line_elems(L), TX = tx_of<R, L>::v;
     constexpr int LPB = 256 / T > 0 ? 256 / T : 1;
     constexpr size_t sm_rows = sizeof(C) * LPB * (L + L / 8), sm_cols = sizeof(C) * L * TX;
+    // rows per block: 256 threads, fewer (down to a warp) while that leaves under two
+    // blocks for each of 152 SMs: x-forward at n = 16 in complex128 was 4 blocks and
+    // 40 us, with 32 it takes 21
+    auto launch_rows = [&](auto kernel, long rows, auto... args) {
+        int lines = LPB;
+        while (lines % 2 == 0 && lines * T >= 64 && (rows + lines - 1) / lines < 2 * 152) lines /= 2;
+        launch_pdl(kernel, dim3((unsigned)((rows + lines - 1) / lines)), dim3(lines * T), sizeof(C) * lines * (L + L / 8), s, args...);
+    };
     const bool fused = (zvar & ZPLAN_FUSED_XY) != 0; // x and y passes fused per z-plane
     zvar &= ZPLAN_FUSED_XY - 1;
     constexpr size_t sm_zprod = sm_cols + sizeof(C) * 4 * n * TX;
@@ -1094,8 +1102,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     }
     if (!fused_done) {
         long rows = (long)nb * n2;
-        launch_pdl(k2_xfwd<R, L>, dim3((unsigned)((rows + LPB - 1) / LPB)), dim3(LPB * T), sm_rows, s, xb, m, p, W1,
-                   (int)rows, tw);
+        launch_rows(k2_xfwd<R, L>, rows, xb, m, p, W1, (int)rows, tw);
         mark();
         if constexpr (line_elems(L) == 8 && n % 2 == 0)
             launch_pdl(k2_cols2<R, L, -1, true>, dim3(L / TX, n / 2, nb * 4), dim3(THR), 2 * sm_cols, s, (const C *)W1,
@@ -1172,8 +1179,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     mark();
     {
         long rows = (long)nb * 3 * n2;
-        launch_pdl(k2_xinv<R, L>, dim3((unsigned)((rows + LPB - 1) / LPB)), dim3(LPB * T), sm_rows, s, (const C *)W1,
-                   xb, yb, rows, tw);
+        launch_rows(k2_xinv<R, L>, rows, (const C *)W1, xb, yb, rows, tw);
     }
     mark();
     return SPM_OK;
