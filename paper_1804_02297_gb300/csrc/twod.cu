@@ -552,6 +552,10 @@ struct Geom2 {
     int rlo[2], rhi[2]; // complement box
 };
 
+struct Geoms2 {
+    Geom2 c[9]; // every class
+};
+
 Geom2 geom2(int cls, int n)
 {
     Geom2 g;
@@ -581,9 +585,13 @@ constexpr int GRAM_UT = 64;      // complement offsets staged per tile
 // three kernels at the class's T neighbourhood offsets o (shared memory), and
 // thread (o, o') accumulates the four sums C_00, C_11, C_12, C_22 of
 // C_ab[o][o'] = sum_u K_a(o - u) conj(K_b(o' - u)), K_0 = G, K_d = G^d, over
-// the tile (u in the neighbourhood box itself is skipped).  part[block][kind][pair].
-__global__ void __launch_bounds__(128) k2_gram(const double2 *__restrict__ E, Geom2 g, int n, double2 *part)
+// the tile (u in the neighbourhood box itself is skipped).  blockIdx.y is the class:
+// part[class][block][kind][pair].
+__global__ void __launch_bounds__(128) k2_gram(const double2 *__restrict__ E, const __grid_constant__ Geoms2 gs, int n,
+                                               double2 *part)
 {
+    const Geom2 &g = gs.c[blockIdx.y];
+    part += (long)blockIdx.y * gridDim.x * 4 * 81;
     __shared__ double2 st[GRAM_UT][9][3];
     const int W = 2 * n - 1;
     const long W2 = (long)W * W;
@@ -625,118 +633,154 @@ __global__ void __launch_bounds__(128) k2_gram(const double2 *__restrict__ E, Ge
         for (int kk = 0; kk < 4; ++kk) part[((long)blockIdx.x * 4 + kk) * 81 + pair] = acc[kk];
 }
 
-// sum the per-block partial Gram sums: out[kind][pair]
+// sum the per-block partial Gram sums: out[class][kind][pair]
 __global__ void k2_gram_sum(const double2 *__restrict__ part, int nblocks, double2 *out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 4 * 81) return;
+    part += (long)blockIdx.y * nblocks * 4 * 81 + i;
     double2 s = make_double2(0, 0);
-    for (int b = 0; b < nblocks; ++b) s = s + part[(long)b * 4 * 81 + i];
-    out[i] = s;
+#pragma unroll 16
+    for (int b = 0; b < nblocks; ++b) s = s + part[(long)b * 4 * 81];
+    out[blockIdx.y * 4 * 81 + i] = s;
 }
 
 __device__ __forceinline__ double2 zm(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
-// One thread per class: H = M M^H from the Gram sums, cyclic Jacobi
-// eigen-decomposition, alpha = conj(eigenvectors of the two smallest
-// eigenvalues), sv = sqrt(eigenvalues) ascending, beta = B^T alpha.
-__global__ void k2_eig(const double2 *__restrict__ part, const double2 *__restrict__ E, Geom2 g, int n, double k,
-                       double2 *alpha, double2 *beta, double *sv)
+// One block per class: H = M M^H from the Gram sums, Jacobi eigen-decomposition,
+// alpha = conj(eigenvectors of the two smallest eigenvalues), sv = sqrt(eigenvalues)
+// ascending, beta = B^T alpha.  A sweep is M - 1 rounds of M/2 disjoint rotations (the
+// round-robin ordering; M = 8, 12, 18): a rotation by one thread costs its FP64
+// instructions one after the other, about 20 us, and a set-up has some 8000 of them (one
+// thread for all of them, class after class, took 0.1 s of a set-up's 0.28 s at n = 119).
+constexpr int EIG2_THREADS = 192; // 9 pairs x 18 rows, in whole warps
+__global__ void __launch_bounds__(EIG2_THREADS) k2_eig(const double2 *__restrict__ sums, const double2 *__restrict__ E,
+                                                       const __grid_constant__ Geoms2 gs, int n, double k, double2 *alpha,
+                                                       double2 *beta, double *sv)
 {
-    // the small dense work sits in shared memory (no large per-thread stack frame)
-    __shared__ double2 Cs[4][81], A[18][18], V[18][18];
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int T = g.T, M = 2 * T;
-    for (int kk = 0; kk < 4; ++kk)
-        for (int pr = 0; pr < T * T; ++pr) Cs[kk][pr] = part[kk * 81 + pr];
+    __shared__ double2 A[18][18], V[18][18], rph[9];
+    __shared__ double rc[9], rs[9], fro;
+    __shared__ int rp[9], rq[9], idx[18];
+    __shared__ unsigned long long off;
+    const Geom2 &g = gs.c[blockIdx.x];
+    sums += blockIdx.x * 4 * 81;
+    alpha += blockIdx.x * 36;
+    beta += blockIdx.x * 54;
+    sv += blockIdx.x * 18;
+    const int T = g.T, M = 2 * T, tid = threadIdx.x, np = M / 2;
     const double k4 = k * k * k * k;
-    for (int r = 0; r < M; ++r)
-        for (int c = 0; c < M; ++c) {
-            const int d = r / T, o = r % T, e = c / T, op = c % T;
-            double2 v;
-            if (d == 0 && e == 0) v = Cs[1][o * T + op];
-            else if (d == 1 && e == 1) v = Cs[3][o * T + op];
-            else if (d == 0 && e == 1) v = Cs[2][o * T + op];
-            else v = conj_of(Cs[2][op * T + o]); // C_21[o][o'] = conj(C_12[o'][o])
-            if (d == e) { v.x += k4 * Cs[0][o * T + op].x; v.y += k4 * Cs[0][o * T + op].y; }
-            A[r][c] = v;
-            V[r][c] = make_double2(r == c ? 1.0 : 0.0, 0.0);
+    for (int e = tid; e < M * M; e += EIG2_THREADS) {
+        const int r = e / M, c = e % M, d = r / T, o = r % T, f = c / T, op = c % T;
+        double2 v;
+        if (d == 0 && f == 0) v = sums[81 + o * T + op];
+        else if (d == 1 && f == 1) v = sums[3 * 81 + o * T + op];
+        else if (d == 0) v = sums[2 * 81 + o * T + op];
+        else v = conj_of(sums[2 * 81 + op * T + o]); // C_21[o][o'] = conj(C_12[o'][o])
+        if (d == f) {
+            v.x += k4 * sums[o * T + op].x;
+            v.y += k4 * sums[o * T + op].y;
         }
-    for (int r = 0; r < M; ++r) A[r][r].y = 0.0;
-    double fro = 0;
-    for (int r = 0; r < M; ++r)
-        for (int c = 0; c < M; ++c) fro += A[r][c].x * A[r][c].x + A[r][c].y * A[r][c].y;
-    for (int sweep = 0; sweep < 60; ++sweep) {
-        double off = 0;
+        if (r == c) v.y = 0.0;
+        A[r][c] = v;
+        V[r][c] = make_double2(r == c ? 1.0 : 0.0, 0.0);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        double s = 0;
         for (int r = 0; r < M; ++r)
-            for (int c = r + 1; c < M; ++c) off += A[r][c].x * A[r][c].x + A[r][c].y * A[r][c].y;
-        if (off <= 1e-34 * fro) break;
-        for (int pp = 0; pp < M; ++pp)
-            for (int q = pp + 1; q < M; ++q) {
-                const double2 cpq = A[pp][q];
-                const double ab = sqrt(cpq.x * cpq.x + cpq.y * cpq.y);
-                if (ab <= 1e-300) continue;
-                const double2 e = make_double2(cpq.x / ab, cpq.y / ab); // phase of A_pq
-                const double zeta = (A[q][q].x - A[pp][pp].x) / (2.0 * ab);
-                const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                const double cs = 1.0 / sqrt(1.0 + t * t), sn = t * cs;
-                // J = diag(1, conj e) * [[cs, sn], [-sn, cs]] on (pp, q): A <- J^H A J, V <- V J
-                const double2 ce = conj_of(e);
-                for (int r = 0; r < M; ++r) { // columns
-                    const double2 ap = A[r][pp], aq = A[r][q];
-                    const double2 aqe = zm(aq, ce);
-                    A[r][pp] = make_double2(cs * ap.x - sn * aqe.x, cs * ap.y - sn * aqe.y);
-                    A[r][q] = make_double2(sn * ap.x + cs * aqe.x, sn * ap.y + cs * aqe.y);
-                    const double2 vp = V[r][pp], vq = V[r][q];
-                    const double2 vqe = zm(vq, ce);
-                    V[r][pp] = make_double2(cs * vp.x - sn * vqe.x, cs * vp.y - sn * vqe.y);
-                    V[r][q] = make_double2(sn * vp.x + cs * vqe.x, sn * vp.y + cs * vqe.y);
+            for (int c = 0; c < M; ++c) s += A[r][c].x * A[r][c].x + A[r][c].y * A[r][c].y;
+        fro = s;
+    }
+    for (int sweep = 0; sweep < 60; ++sweep) {
+        if (tid == 0) off = 0ull;
+        __syncthreads();
+        for (int round = 0; round < M - 1; ++round) {
+            if (tid < np) {
+                const int pb = M - 1 - tid;
+                int p = tid == 0 ? 0 : (tid - 1 + round) % (M - 1) + 1, q = (pb - 1 + round) % (M - 1) + 1;
+                if (p > q) { const int s = p; p = q; q = s; }
+                const double2 b = A[p][q];
+                const double b2 = b.x * b.x + b.y * b.y, ab = sqrt(b2);
+                double cs = 1.0, sn = 0.0;
+                double2 ph = make_double2(1.0, 0.0);
+                if (ab > 1e-300) {
+                    atomicMax(&off, (unsigned long long)__double_as_longlong(b2)); // positive doubles order as integers
+                    const double zeta = (A[q][q].x - A[p][p].x) / (2.0 * ab);
+                    const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+                    cs = 1.0 / sqrt(1.0 + t * t);
+                    sn = t * cs;
+                    ph = make_double2(b.x / ab, -b.y / ab); // conj of the phase of A_pq
                 }
-                for (int c = 0; c < M; ++c) { // rows
-                    const double2 ap = A[pp][c], aq = A[q][c];
-                    const double2 aqe = zm(aq, e);
-                    A[pp][c] = make_double2(cs * ap.x - sn * aqe.x, cs * ap.y - sn * aqe.y);
-                    A[q][c] = make_double2(sn * ap.x + cs * aqe.x, sn * ap.y + cs * aqe.y);
-                }
-                A[pp][q] = A[q][pp] = make_double2(0.0, 0.0);
-                A[pp][pp].y = A[q][q].y = 0.0;
+                rp[tid] = p;
+                rq[tid] = q;
+                rc[tid] = cs;
+                rs[tid] = sn;
+                rph[tid] = ph;
             }
+            __syncthreads();
+            // J = diag(1, ph) [[cs, sn], [-sn, cs]] on each (p, q): A <- J^H A J, V <- V J
+            const int j = tid / M, i = tid % M;
+            const bool act = j < np;
+            const int p = act ? rp[j] : 0, q = act ? rq[j] : 0;
+            const double cs = act ? rc[j] : 1.0, sn = act ? rs[j] : 0.0;
+            const double2 ph = act ? rph[j] : make_double2(1.0, 0.0);
+            if (act) { // columns
+                const double2 ap = A[i][p], aq = zm(A[i][q], ph);
+                A[i][p] = make_double2(cs * ap.x - sn * aq.x, cs * ap.y - sn * aq.y);
+                A[i][q] = make_double2(sn * ap.x + cs * aq.x, sn * ap.y + cs * aq.y);
+                const double2 vp = V[i][p], vq = zm(V[i][q], ph);
+                V[i][p] = make_double2(cs * vp.x - sn * vq.x, cs * vp.y - sn * vq.y);
+                V[i][q] = make_double2(sn * vp.x + cs * vq.x, sn * vp.y + cs * vq.y);
+            }
+            __syncthreads();
+            if (act) { // rows; the rotated pair becomes exactly diagonal
+                const double2 ap = A[p][i], aq = zm(A[q][i], conj_of(ph));
+                double2 np_ = make_double2(cs * ap.x - sn * aq.x, cs * ap.y - sn * aq.y);
+                double2 nq_ = make_double2(sn * ap.x + cs * aq.x, sn * ap.y + cs * aq.y);
+                if (i == p) { np_.y = 0.0; nq_ = make_double2(0.0, 0.0); }
+                if (i == q) { nq_.y = 0.0; np_ = make_double2(0.0, 0.0); }
+                A[p][i] = np_;
+                A[q][i] = nq_;
+            }
+            __syncthreads();
+        }
+        // the sum over all pairs is at most M (M - 1) / 2 times the largest
+        const bool done = __longlong_as_double((long long)off) * (M * (M - 1) / 2) <= 1e-34 * fro;
+        __syncthreads();
+        if (done) break;
     }
-    int idx[18];
-    for (int i = 0; i < M; ++i) idx[i] = i;
-    for (int i = 1; i < M; ++i) { // insertion sort by eigenvalue
-        const int v = idx[i];
-        int j = i - 1;
-        while (j >= 0 && A[idx[j]][idx[j]].x > A[v][v].x) { idx[j + 1] = idx[j]; --j; }
-        idx[j + 1] = v;
+    if (tid == 0) {
+        for (int i = 0; i < M; ++i) idx[i] = i;
+        for (int i = 1; i < M; ++i) { // insertion sort by eigenvalue
+            const int v = idx[i];
+            int j = i - 1;
+            while (j >= 0 && A[idx[j]][idx[j]].x > A[v][v].x) { idx[j + 1] = idx[j]; --j; }
+            idx[j + 1] = v;
+        }
     }
-    for (int i = 0; i < 18; ++i) sv[i] = i < M ? sqrt(fmax(A[idx[i]][idx[i]].x, 0.0)) : 0.0;
-    for (int r = 0; r < 18; ++r)
-        for (int c = 0; c < 2; ++c) alpha[r * 2 + c] = r < M ? conj_of(V[r][idx[c]]) : make_double2(0.0, 0.0);
+    __syncthreads();
+    if (tid < 18) sv[tid] = tid < M ? sqrt(fmax(A[idx[tid]][idx[tid]].x, 0.0)) : 0.0;
+    if (tid < 36) alpha[tid] = tid / 2 < M ? conj_of(V[tid / 2][idx[tid % 2]]) : make_double2(0.0, 0.0);
     // beta[(f,o'),c] = sum_{(d,o)} alpha[(d,o),c] K_{(d,o),(f,o')}
     const int W = 2 * n - 1;
     const long W2 = (long)W * W;
     const double k2 = k * k;
-    for (int r = 0; r < 27; ++r)
-        for (int c = 0; c < 2; ++c) beta[r * 2 + c] = make_double2(0.0, 0.0);
-    for (int f = 0; f < 3; ++f)
-        for (int op = 0; op < T; ++op)
-            for (int c = 0; c < 2; ++c) {
-                double2 s = make_double2(0.0, 0.0);
-                for (int d = 0; d < 2; ++d)
-                    for (int o = 0; o < T; ++o) {
-                        const long e = (long)(g.off[o][1] - g.off[op][1] + n - 1) * W + (g.off[o][0] - g.off[op][0] + n - 1);
-                        double2 K;
-                        if (f < 2) {
-                            if (f != d) continue;
-                            K = make_double2(k2 * E[e].x, k2 * E[e].y);
-                        } else {
-                            K = E[(1 + d) * W2 + e];
-                        }
-                        s = cfma(alpha[(d * T + o) * 2 + c], K, s);
-                    }
-                beta[(f * T + op) * 2 + c] = s;
+    for (int e = tid; e < 54; e += EIG2_THREADS) {
+        const int r = e / 2, c = e % 2, f = r / T, op = r % T;
+        double2 s = make_double2(0.0, 0.0);
+        if (f < 3) {
+            for (int d = 0; d < 2; ++d) {
+                if (f < 2 && f != d) continue;
+                for (int o = 0; o < T; ++o) {
+                    const long at = (long)(g.off[o][1] - g.off[op][1] + n - 1) * W + (g.off[o][0] - g.off[op][0] + n - 1);
+                    double2 K = E[(f < 2 ? 0 : 1 + d) * W2 + at];
+                    if (f < 2) K = make_double2(k2 * K.x, k2 * K.y);
+                    s = cfma(conj_of(V[d * T + o][idx[c]]), K, s);
+                }
             }
+        }
+        beta[e] = s;
+    }
 }
 
 } // namespace
@@ -860,19 +904,17 @@ spm_status fit_stencils(spm2_problem_s *P)
     const int n = P->n;
     cudaStream_t s = P->stream;
     DevBuf part, out;
-    SPM_TRY(part.ensure(sizeof(double2) * (GRAM_BLOCKS + 1) * 4 * 81));
-    double2 *sums = part.as<double2>() + (long)GRAM_BLOCKS * 4 * 81;
+    SPM_TRY(part.ensure(sizeof(double2) * 9 * (GRAM_BLOCKS + 1) * 4 * 81));
+    double2 *sums = part.as<double2>() + 9L * GRAM_BLOCKS * 4 * 81;
     SPM_TRY(out.ensure(sizeof(double2) * 9 * (18 + 27) * 2 + sizeof(double) * 9 * 18));
     double2 *al = out.as<double2>(), *be = al + 9 * 18 * 2;
     double *sv = reinterpret_cast<double *>(be + 9 * 27 * 2);
-    for (int cls = 0; cls < 9; ++cls) {
-        const Geom2 g = geom2(cls, n);
-        k2_gram<<<GRAM_BLOCKS, 128, 0, s>>>(P->entries.as<double2>(), g, n, part.as<double2>());
-        k2_gram_sum<<<3, 128, 0, s>>>(part.as<double2>(), GRAM_BLOCKS, sums);
-        k2_eig<<<1, 32, 0, s>>>(sums, P->entries.as<double2>(), g, n, P->k, al + cls * 36, be + cls * 54,
-                                sv + cls * 18);
-        SPM_CUDA_TRY(cudaGetLastError());
-    }
+    Geoms2 gs;
+    for (int cls = 0; cls < 9; ++cls) gs.c[cls] = geom2(cls, n);
+    k2_gram<<<dim3(GRAM_BLOCKS, 9), 128, 0, s>>>(P->entries.as<double2>(), gs, n, part.as<double2>());
+    k2_gram_sum<<<dim3(3, 9), 128, 0, s>>>(part.as<double2>(), GRAM_BLOCKS, sums);
+    k2_eig<<<9, EIG2_THREADS, 0, s>>>(sums, P->entries.as<double2>(), gs, n, P->k, al, be, sv);
+    SPM_CUDA_TRY(cudaGetLastError());
     P->alpha_h.resize(9 * 18 * 2 * 2);
     P->beta_h.resize(9 * 27 * 2 * 2);
     P->sv_h.resize(9 * 18);
