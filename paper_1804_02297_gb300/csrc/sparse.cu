@@ -84,15 +84,34 @@ __global__ void k_front_assemble(C *F, int f, const C *__restrict__ S, const int
     }
 }
 
-// ---- batched small fronts: one block per front, the whole front in shared memory
-// A front of f unknowns (o3 own first) is assembled from S and the children's
-// updates, then swept by Gauss-Jordan over its o3 own pivots with partial
-// pivoting among the own rows (explicit row swaps) and the static pivot floor:
-// after the sweep the front holds [(P F11)^-1, F11^-1 F12; -F21 (P F11)^-1,
-// F22 - F21 F11^-1 F12], from which G = [F11^-1; F21 F11^-1] (columns put back
-// in place), X = F11^-1 F12 and the update F22 - F21 X are written out.  The
-// same quantities as the per-front path (dense inverse + GEMMs), in one launch
-// for every small front of a tree level.
+// ---- batched fronts: a level's fronts advance together, panel by panel
+// A front of f unknowns (o3 own first) is assembled from S and the children's updates,
+// then swept by Gauss-Jordan over its o3 own pivots with partial pivoting among the own
+// rows (row swaps) and the static pivot floor: after the sweep the front holds
+// [(P F11)^-1, F11^-1 F12; -F21 (P F11)^-1, F22 - F21 F11^-1 F12], from which
+// G = [F11^-1; F21 F11^-1] (columns put back in place), X = F11^-1 F12 and the update
+// F22 - F21 X are stored: the same quantities as the per-front path (dense inverse and
+// GEMMs).  Every front of a level lies in global scratch and takes one panel of BP_NB
+// pivots at a time, K its rows and columns:
+//   k_bp_panel   (a block per front) the steps on the unpivoted own rows of the panel's
+//                columns, in shared memory
+//   k_bp_cross   the same steps on the other rows of the panel's columns, and on the
+//                pivot rows of the other columns (where it also swaps the rows)
+//   k_bp_update  the same steps on everything else: A[i][j] -= M[i][:] S[:][j]
+// Step jj divides the pivot row by the pivot and subtracts the row's multiple M[i][jj]
+// (the entry of the pivot's column before the step) from every other row i.  The first
+// two kernels keep the multipliers M (moved along by later row swaps) and the scaled pivot
+// rows S as each step leaves them, so every entry of the front sees the same operations in
+// the same order as in an unblocked sweep.  (Forming P^-1 of the pivot block and adding the product
+// of M P^-1 and the pivot rows is the same work in fewer steps, but its factors' probe
+// residuals were 1.3 to 2 times as large.)
+// Bound: the FP64 pipe for complex128 (4 o3 f^2 FMAs; two lanes per SM) and the chain of
+// pivots.  With one block per front, the few fronts near the root had one SM each: of
+// the 204 ms of a 2-D factor at n = 119 the last five levels took 192.  Spread over the
+// chip the factor takes 14 ms (n = 239: 361 -> 137; 3-D complex64 n = 16: 86 -> 12,
+// n = 32: 406 -> 231, n = 64: 5.5 -> 4.8 s; 3-D complex128 n = 16: 338 -> 79 ms).  At
+// n = 119 the updates take 6 ms of it (their FP64 work alone 3.2), the panels' chains 3.2
+// (4 us a pivot), k_bp_cross 1.2.
 struct BatchFront {
     int own_off, nown, map_off, e0, e1, e2, ew0, ew1, f, o3, nch;
     int ch_bc[2], ch_rel[2];
@@ -101,51 +120,62 @@ struct BatchFront {
     const void *ch_upd[2];
 };
 
-template <typename C> __device__ __forceinline__ C bdiv(C a, C b)
+constexpr int BP_NB = 8, BP_THREADS = 256;
+template <typename C> struct BatchPanel {
+    C prow[BP_NB][BP_NB];               // scaled pivot row of each step ([jj][jj]: 1 / pivot)
+    int nmove;                          // rows the panel's swaps gave new contents
+    int dst[2 * BP_NB], src[2 * BP_NB]; // the first are the pivot rows
+};
+
+// The sweep's arithmetic, rounding fixed: a - m b with the product first (six FP64
+// instructions where chained FMAs would be four, but the factors' residuals are smaller,
+// 0.85 of the others' in 3-D complex64), m b, and |d|^2.  A box of the dissection that is
+// nearly singular magnifies the last bit of any of these to 1e-8 in S^-1, so the kernels
+// must not leave the contraction to each one's context.
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+template <typename C> __device__ __forceinline__ C csub_mul(C a, C m, C b)
 {
-    using R = decltype(a.x);
-    const R d = b.x * b.x + b.y * b.y;
+    a.x -= fma(m.x, b.x, -mul_rn(m.y, b.y));
+    a.y -= fma(m.y, b.x, mul_rn(m.x, b.y));
+    return a;
+}
+template <typename C> __device__ __forceinline__ C cmul_rn(C a, C b)
+{
     C r;
-    r.x = (a.x * b.x + a.y * b.y) / d;
-    r.y = (a.y * b.x - a.x * b.y) / d;
+    r.x = fma(a.x, b.x, -mul_rn(a.y, b.y));
+    r.y = fma(a.x, b.y, mul_rn(a.y, b.x));
     return r;
 }
-
-template <typename C>
-__global__ void __launch_bounds__(256) k_front_batch(const BatchFront *__restrict__ fronts, const C *__restrict__ S,
-                                                     const int *__restrict__ pts, const int *__restrict__ maps,
-                                                     const int *__restrict__ rels, GridDesc g, C *fac, double tau,
-                                                     int *raised, C *gscratch, long gstride)
+template <typename C> __device__ __forceinline__ C neg_mul(C m, C b)
 {
-    using R = decltype(C{}.x);
-    extern __shared__ unsigned char smem_raw[];
+    C r = cmul_rn(m, b);
+    r.x = -r.x;
+    r.y = -r.y;
+    return r;
+}
+template <typename C> __device__ __forceinline__ auto norm2_rn(C a) { return fma(a.x, a.x, mul_rn(a.y, a.y)); }
+
+// F (zeroed) <- the front's entries of S
+template <typename C>
+__global__ void __launch_bounds__(BP_THREADS) k_bp_assemble(const BatchFront *__restrict__ fronts, const C *__restrict__ S,
+                                                            const int *__restrict__ pts, const int *__restrict__ maps,
+                                                            GridDesc g, C *scratch, long stride, int *perm, int permld)
+{
+    pdl_wait_and_trigger();
     const BatchFront fr = fronts[blockIdx.x];
-    const int f = fr.f, o3 = fr.o3, b3 = f - o3;
-    // the front, f x f column-major (row r, column c at c * f + r): in shared memory,
-    // or for larger fronts in this block's slice of a global scratch (then only the
-    // pivot row, pivot column and permutation sit in shared memory)
-    C *F = gscratch ? gscratch + (long)blockIdx.x * gstride : reinterpret_cast<C *>(smem_raw);
-    C *prow = gscratch ? reinterpret_cast<C *>(smem_raw) : F + (long)f * f; // the scaled pivot row
-    C *pcol = prow + f;                     // the pivot column before the step
-    int *perm = reinterpret_cast<int *>(pcol + f);
-    __shared__ R red_v[8];
-    __shared__ R s_floor;
-    __shared__ int s_p;
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
-    for (int i = tid; i < f * f; i += nt) F[i] = czero<C>();
-    for (int i = tid; i < o3; i += nt) perm[i] = i;
-    __syncthreads();
-    const int D = g.D, DD = g.D * g.D;
+    C *F = scratch + (long)blockIdx.x * stride;
+    const int f = fr.f, D = g.D, DD = g.D * g.D, first = blockIdx.y * blockDim.x + threadIdx.x, step = gridDim.y * blockDim.x;
     const int *own_pts = pts + fr.own_off, *lmap = maps + fr.map_off;
-    for (int gid = tid; gid < fr.nown * g.nsten; gid += nt) {
+    for (int i = first; i < fr.o3; i += step) perm[(long)blockIdx.x * permld + i] = i;
+    for (int gid = first; gid < fr.nown * g.nsten; gid += step) {
         const int a = gid / g.nsten, s = gid % g.nsten;
         const int o1 = s % 3 - 1, o2 = (s / 3) % 3 - 1, oz = g.nsten == 27 ? s / 9 - 1 : 0;
         const int i = own_pts[a];
-        const int i1 = i % g.n1, i2 = (i / g.n1) % g.n2, i3 = i / (g.n1 * g.n2);
-        const int j1 = i1 + o1, j2 = i2 + o2, j3 = i3 + oz;
+        const int j1 = i % g.n1 + o1, j2 = (i / g.n1) % g.n2 + o2, j3 = i / (g.n1 * g.n2) + oz;
         if (j1 < 0 || j2 < 0 || j3 < 0 || j1 >= g.n1 || j2 >= g.n2 || j3 >= g.n3) continue;
         const int lj = lmap[((j3 - fr.e2) * fr.ew1 + (j2 - fr.e1)) * fr.ew0 + (j1 - fr.e0)];
-        if (lj < 0) continue;
+        if (lj < 0) continue; // eliminated in a child
         const long j = ((long)j3 * g.n2 + j2) * g.n1 + j1;
         const C *blk = S + ((long)i * g.nsten + s) * DD;
         for (int c = 0; c < D; ++c)
@@ -156,110 +186,312 @@ __global__ void __launch_bounds__(256) k_front_batch(const BatchFront *__restric
                 for (int q = 0; q < D; ++q) F[(long)(D * a + q) * f + D * lj + c] = bj[c * D + q];
         }
     }
-    __syncthreads();
-    for (int ch = 0; ch < fr.nch; ++ch) { // children one after the other: their maps overlap
-        const C *U = reinterpret_cast<const C *>(fr.ch_upd[ch]);
-        const int bc = fr.ch_bc[ch];
-        const int *rel = rels + fr.ch_rel[ch];
-        for (int e = tid; e < bc * bc; e += nt) {
-            const C u = U[e];
-            C &d = F[(long)rel[e / bc] * f + rel[e % bc]];
+}
+
+// F += the update of child ch (the children one after the other: their maps overlap)
+template <typename C>
+__global__ void __launch_bounds__(BP_THREADS) k_bp_extend(const BatchFront *__restrict__ fronts, int ch,
+                                                          const int *__restrict__ rels, C *scratch, long stride)
+{
+    pdl_wait_and_trigger();
+    const BatchFront &fr = fronts[blockIdx.x];
+    if (ch >= fr.nch) return;
+    C *F = scratch + (long)blockIdx.x * stride;
+    const C *U = reinterpret_cast<const C *>(fr.ch_upd[ch]);
+    const int bc = fr.ch_bc[ch], f = fr.f;
+    const int *rel = rels + fr.ch_rel[ch];
+    for (int c = blockIdx.y; c < bc; c += gridDim.y) {
+        C *col = F + (long)rel[c] * f;
+        for (int r = threadIdx.x; r < bc; r += BP_THREADS) {
+            const C u = U[(long)c * bc + r];
+            C d = col[rel[r]];
             d.x += u.x;
             d.y += u.y;
+            col[rel[r]] = d;
         }
-        __syncthreads();
     }
-    // pivot floor: tau times the largest |entry| of F11
-    R mx = 0;
-    for (int e = tid; e < o3 * o3; e += nt) {
-        const C a = F[(long)(e / o3) * f + e % o3];
-        mx = max(mx, a.x * a.x + a.y * a.y);
-    }
+}
+
+// amax2[front] = the largest |entry|^2 of F11, as the bits of a double (zeroed before)
+template <typename C>
+__global__ void __launch_bounds__(BP_THREADS) k_bp_absmax(const BatchFront *__restrict__ fronts, const C *scratch, long stride,
+                                                          unsigned long long *amax2)
+{
+    pdl_wait_and_trigger();
+    const int f = fronts[blockIdx.x].f, o3 = fronts[blockIdx.x].o3;
+    const C *F = scratch + (long)blockIdx.x * stride;
+    unsigned long long mx = 0;
+    for (int c = blockIdx.y; c < o3; c += gridDim.y)
+        for (int r = threadIdx.x; r < o3; r += BP_THREADS) {
+            const C a = F[(long)c * f + r];
+            mx = max(mx, (unsigned long long)__double_as_longlong((double)norm2_rn(a)));
+        }
     for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) red_v[wid] = mx;
+    if ((threadIdx.x & 31) == 0 && mx) atomicMax(&amax2[blockIdx.x], mx);
+}
+
+// A step's rows x BP_NB entries are spread over the block: thread t takes row t % rows and
+// the columns of group t / rows.  M: [front][BP_NB][fm].
+template <typename C>
+__global__ void __launch_bounds__(BP_THREADS) k_bp_panel(const BatchFront *__restrict__ fronts, C *scratch, long stride, int k0,
+                                                         double tau, const unsigned long long *__restrict__ amax2, int *perm,
+                                                         int permld, C *M, int fm, BatchPanel<C> *panels, int *raised)
+{
+    using R = decltype(C{}.x);
+    pdl_wait_and_trigger();
+    const int f = fronts[blockIdx.x].f, o3 = fronts[blockIdx.x].o3;
+    if (k0 >= o3) return;
+    const int kb = min(BP_NB, o3 - k0), m = o3 - k0;
+    extern __shared__ unsigned char smem_raw[];
+    C *P = reinterpret_cast<C *>(smem_raw); // [BP_NB][m]
+    C *pc = P + BP_NB * m;                  // [m] the step's column before elimination
+    __shared__ C prow[BP_NB];
+    __shared__ unsigned long long cand[BP_THREADS / 32];
+    __shared__ int candi[BP_THREADS / 32], pivs[BP_NB];
+    C *F = scratch + (long)blockIdx.x * stride + k0;
+    C *Mf = M + (long)blockIdx.x * BP_NB * fm + k0;
+    BatchPanel<C> &bp = panels[blockIdx.x];
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
+    for (int e = tid; e < kb * m; e += nt) P[e] = F[(long)(k0 + e / m) * f + e % m];
+    const R fl = (R)(tau * sqrt(__longlong_as_double((long long)amax2[blockIdx.x])));
+    // column groups: 1, 2, 4 or 8, as many as give every thread work
+    int gr = 1;
+    while (gr < BP_NB && m * gr * 2 <= nt) gr *= 2;
+    const int cw = BP_NB / gr, rows = gr == 1 ? nt : m, r0 = tid % rows, cg = tid / rows * cw;
     __syncthreads();
-    if (tid == 0) {
-        R m2 = red_v[0];
-        for (int w = 1; w < nt / 32; ++w) m2 = max(m2, red_v[w]);
-        s_floor = (R)(tau * sqrt((double)m2));
+    for (int jj = 0; jj < kb; ++jj) {
+        // the largest |P[jj][i]| over the unpivoted own rows, the lowest row on ties;
+        // magnitudes compared as the bits of non-negative doubles
+        unsigned long long best = 0;
+        int bi = m;
+        for (int i = tid; i < m; i += nt) {
+            const C a = P[jj * m + i];
+            pc[i] = a;
+            if (i < jj) continue;
+            const unsigned long long v = (unsigned long long)__double_as_longlong((double)norm2_rn(a));
+            if (v > best || bi == m) { best = v; bi = i; }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, o);
+            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+            if (oi < m && (bi == m || ov > best || (ov == best && oi < bi))) { best = ov; bi = oi; }
+        }
+        if (lane == 0) { cand[wid] = best; candi[wid] = bi; }
+        __syncthreads();
+        if (wid == 0) {
+            best = cand[0];
+            bi = candi[0];
+            for (int w = 1; w < nt / 32; ++w)
+                if (candi[w] < m && (bi == m || cand[w] > best || (cand[w] == best && candi[w] < bi))) { best = cand[w]; bi = candi[w]; }
+            const int p = bi;
+            // the pivot row, divided by the (floored) pivot; rows p and jj change places
+            C v = czero<C>();
+            if (lane < kb) {
+                v = P[lane * m + p];
+                P[lane * m + p] = P[lane * m + jj];
+            }
+            C d;
+            d.x = __shfl_sync(0xffffffffu, v.x, jj);
+            d.y = __shfl_sync(0xffffffffu, v.y, jj);
+            R d2 = norm2_rn(d);
+            if (d2 < fl * fl) { // the static pivot floor
+                const R ad = sqrt(d2);
+                const R sx = ad > 0 ? d.x / ad : (R)1, sy = ad > 0 ? d.y / ad : (R)0;
+                d.x = fl * sx;
+                d.y = fl * sy;
+                d2 = norm2_rn(d);
+                if (lane == 0) atomicAdd(raised, 1);
+            }
+            // conj(d) / |d|^2: the two divisions in two lanes at once
+            const R quo = (lane & 1 ? -d.y : d.x) / d2;
+            C inv_d;
+            inv_d.x = __shfl_sync(0xffffffffu, quo, 0);
+            inv_d.y = __shfl_sync(0xffffffffu, quo, 1);
+            if (lane < kb) {
+                const C w = lane == jj ? inv_d : cmul_rn(v, inv_d);
+                prow[lane] = w;
+                bp.prow[jj][lane] = w;
+            }
+            if (lane == 0) {
+                pivs[jj] = p;
+                pc[p] = pc[jj];
+            }
+        }
+        __syncthreads();
+        if (r0 < m && cg < kb) {
+            for (int i = r0; i < m; i += rows) {
+                const C a = pc[i];
+                if (cg == 0) Mf[jj * fm + i] = a;
+#pragma unroll 1
+                for (int c = cg; c < min(cg + cw, kb); ++c)
+                    P[c * m + i] = i == jj ? prow[c] : (c == jj ? neg_mul(a, prow[jj]) : csub_mul(P[c * m + i], a, prow[c]));
+            }
+        }
+        if (wid == nt / 32 - 1 && lane < jj && pivs[jj] != jj) { // the swapped rows' earlier multipliers
+            C *u = Mf + lane * fm + jj, *w = Mf + lane * fm + pivs[jj];
+            const C t = *u;
+            *u = *w;
+            *w = t;
+        }
+        __syncthreads();
+    }
+    for (int e = tid; e < kb * m; e += nt) F[(long)(k0 + e / m) * f + e % m] = P[e];
+    if (tid == 0) { // the rows whose contents the swaps moved
+        int nmove = kb;
+        for (int jj = 0; jj < kb; ++jj) bp.dst[jj] = bp.src[jj] = k0 + jj;
+        int *pm = perm + (long)blockIdx.x * permld;
+        for (int jj = 0; jj < kb; ++jj) {
+            const int p = k0 + pivs[jj];
+            if (p == k0 + jj) continue;
+            const int t = pm[p];
+            pm[p] = pm[k0 + jj];
+            pm[k0 + jj] = t;
+            int q = 0;
+            while (q < nmove && bp.dst[q] != p) ++q;
+            if (q == nmove) {
+                bp.dst[q] = bp.src[q] = p;
+                ++nmove;
+            }
+            const int u = bp.src[q];
+            bp.src[q] = bp.src[jj];
+            bp.src[jj] = u;
+        }
+        bp.nmove = nmove;
+    }
+}
+
+// blockIdx.y < row_blocks: the panel's columns on the other rows (pivoted before, and
+// boundary), eight rows and four column groups per warp, the step's multiplier passed
+// between the groups.  The other blocks: the pivot rows of the other columns, a thread per
+// (pivot row, column): the panel's row swaps first, then the steps, S kept.
+constexpr int BX_THREADS = 128, BX_ROWS = BX_THREADS / 4, BX_COLS = BX_THREADS / BP_NB;
+template <typename C>
+__global__ void __launch_bounds__(BX_THREADS) k_bp_cross(const BatchFront *__restrict__ fronts, C *scratch, long stride, int k0,
+                                                         int row_blocks, C *M, C *S, int fm,
+                                                         const BatchPanel<C> *__restrict__ panels)
+{
+    constexpr int CW = BP_NB / 4;
+    pdl_wait_and_trigger();
+    const int f = fronts[blockIdx.x].f, o3 = fronts[blockIdx.x].o3;
+    if (k0 >= o3) return;
+    const int kb = min(BP_NB, o3 - k0);
+    const BatchPanel<C> &bp = panels[blockIdx.x];
+    C *F = scratch + (long)blockIdx.x * stride;
+    C *Mf = M + (long)blockIdx.x * BP_NB * fm;
+    if ((int)blockIdx.y < row_blocks) {
+        if (blockIdx.y * BX_ROWS >= f - (o3 - k0)) return;
+        const int lane = threadIdx.x & 31, g = lane >> 3;
+        const int e = blockIdx.y * BX_ROWS + (threadIdx.x >> 5) * 8 + (lane & 7), i = e < k0 ? e : e + o3 - k0;
+        F += (long)k0 * f;
+        C a[CW];
+#pragma unroll
+        for (int c = 0; c < CW; ++c) a[c] = g * CW + c < kb && i < f ? F[(long)(g * CW + c) * f + i] : czero<C>();
+#pragma unroll
+        for (int jj = 0; jj < BP_NB; ++jj) {
+            if (jj >= kb) break;
+            C w;
+            w.x = __shfl_sync(0xffffffffu, a[jj % CW].x, (jj / CW) * 8 + (lane & 7));
+            w.y = __shfl_sync(0xffffffffu, a[jj % CW].y, (jj / CW) * 8 + (lane & 7));
+            if (g == 0 && i < f) Mf[jj * fm + i] = w;
+#pragma unroll
+            for (int c = 0; c < CW; ++c)
+                if (g * CW + c < kb) a[c] = g * CW + c == jj ? neg_mul(w, bp.prow[jj][jj]) : csub_mul(a[c], w, bp.prow[jj][g * CW + c]);
+        }
+        if (i >= f) return;
+#pragma unroll
+        for (int c = 0; c < CW; ++c)
+            if (g * CW + c < kb) F[(long)(g * CW + c) * f + i] = a[c];
+        return;
+    }
+    const int c0 = (blockIdx.y - row_blocks) * BX_COLS;
+    if (c0 >= f - kb) return;
+    __shared__ C sr[BP_NB][BX_COLS];
+    const int k = threadIdx.x / BX_COLS, c = threadIdx.x % BX_COLS;
+    const bool act = k < kb && c0 + c < f - kb;
+    const int j = c0 + c < k0 ? c0 + c : c0 + c + kb; // the column
+    C *col = F + (long)j * f;
+    const int q = kb + k; // a displaced row, if there are as many (at most kb)
+    const bool dis = c0 + c < f - kb && q < bp.nmove;
+    C r = act ? col[bp.src[k]] : czero<C>(), away = dis ? col[bp.src[q]] : czero<C>(), mk[BP_NB];
+#pragma unroll
+    for (int jj = 0; jj < BP_NB; ++jj) mk[jj] = act && jj < kb ? Mf[jj * fm + k0 + k] : czero<C>();
+    const C inv = act ? bp.prow[k][k] : czero<C>();
+    __syncthreads(); // every source row has been read
+    if (dis) col[bp.dst[q]] = away;
+#pragma unroll
+    for (int jj = 0; jj < BP_NB; ++jj) {
+        if (jj >= kb) break;
+        if (act && k == jj) {
+            r = cmul_rn(r, inv);
+            sr[jj][c] = r;
+            S[((long)blockIdx.x * fm + j) * BP_NB + jj] = r;
+        }
+        __syncthreads();
+        if (act && k != jj) r = csub_mul(r, mk[jj], sr[jj][c]);
+    }
+    if (act) col[k0 + k] = r;
+}
+
+template <typename C, int CT>
+__global__ void __launch_bounds__(BP_THREADS, 2) k_bp_update(const BatchFront *__restrict__ fronts, C *scratch, long stride,
+                                                          int k0, const C *__restrict__ M, const C *__restrict__ S, int fm)
+{
+    pdl_wait_and_trigger();
+    const int f = fronts[blockIdx.x].f, o3 = fronts[blockIdx.x].o3;
+    if (k0 >= o3) return;
+    const int kb = min(BP_NB, o3 - k0), c0 = blockIdx.y * CT, nc = min(CT, f - kb - c0);
+    if (nc <= 0) return;
+    __shared__ C sr[CT][BP_NB];
+    C *F = scratch + (long)blockIdx.x * stride;
+    const C *Mf = M + (long)blockIdx.x * BP_NB * fm;
+    auto col = [&](int c) { return c0 + c < k0 ? c0 + c : c0 + c + kb; };
+    for (int e = threadIdx.x; e < CT * BP_NB; e += blockDim.x) {
+        const int c = e / BP_NB, q = e % BP_NB;
+        sr[c][q] = c < nc && q < kb ? S[((long)blockIdx.x * fm + col(c)) * BP_NB + q] : czero<C>();
     }
     __syncthreads();
-    const R fl = s_floor;
-    C one;
-    one.x = 1;
-    one.y = 0;
-    for (int k = 0; k < o3; ++k) {
-        if (wid == 0) { // the largest |F[i][k]| over the unpivoted own rows, lowest row on ties
-            R best = -1;
-            int bi = -1;
-            for (int i = k + lane; i < o3; i += 32) {
-                const C a = F[(long)k * f + i];
-                const R v = a.x * a.x + a.y * a.y;
-                if (v > best) { best = v; bi = i; }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                const R ov = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ov > best || (ov == best && oi >= 0 && (bi < 0 || oi < bi))) { best = ov; bi = oi; }
-            }
-            if (lane == 0) s_p = bi;
+    for (int i = threadIdx.x; i < f; i += blockDim.x) {
+        if (i >= k0 && i < k0 + kb) continue;
+        C t[BP_NB];
+#pragma unroll
+        for (int q = 0; q < BP_NB; ++q) t[q] = q < kb ? Mf[q * fm + i] : czero<C>();
+#pragma unroll 2
+        for (int c = 0; c < nc; ++c) {
+            C *at = F + (long)col(c) * f + i;
+            C a = *at;
+#pragma unroll
+            for (int q = 0; q < BP_NB; ++q)
+                if (q < kb) a = csub_mul(a, t[q], sr[c][q]);
+            *at = a;
         }
-        __syncthreads();
-        const int p = s_p;
-        if (p != k) {
-            for (int c = tid; c < f; c += nt) {
-                const C t = F[(long)c * f + p];
-                F[(long)c * f + p] = F[(long)c * f + k];
-                F[(long)c * f + k] = t;
-            }
-            if (tid == 0) { const int t = perm[p]; perm[p] = perm[k]; perm[k] = t; }
-            __syncthreads();
-        }
-        C d = F[(long)k * f + k];
-        const R ad2 = d.x * d.x + d.y * d.y;
-        if (ad2 < fl * fl) { // the static pivot floor
-            const R ad = sqrt(ad2);
-            const R sx = ad > 0 ? d.x / ad : (R)1, sy = ad > 0 ? d.y / ad : (R)0;
-            d.x = fl * sx;
-            d.y = fl * sy;
-            if (tid == 0) atomicAdd(raised, 1);
-        }
-        const C inv_d = bdiv(one, d);
-        for (int j = tid; j < f; j += nt) {
-            prow[j] = j == k ? inv_d : cmul(F[(long)j * f + k], inv_d);
-            pcol[j] = F[(long)k * f + j];
-        }
-        __syncthreads();
-        for (int e = tid; e < f * f; e += nt) {
-            const int i = e % f, j = e / f;
-            C v;
-            if (i == k) {
-                v = prow[j];
-            } else if (j == k) {
-                v = cmul(pcol[i], inv_d);
-                v.x = -v.x;
-                v.y = -v.y;
+    }
+}
+
+// the swept fronts -> G = [F11^-1; F21 F11^-1] (columns put back in place), X, update
+template <typename C>
+__global__ void __launch_bounds__(BP_THREADS) k_bp_store(const BatchFront *__restrict__ fronts, const C *scratch, long stride,
+                                                         const int *__restrict__ perm, int permld, C *fac)
+{
+    pdl_wait_and_trigger();
+    const BatchFront &fr = fronts[blockIdx.x];
+    const C *F = scratch + (long)blockIdx.x * stride;
+    const int f = fr.f, o3 = fr.o3, b3 = f - o3;
+    C *G = fac + fr.fac_off, *X = G + (long)f * o3, *U = reinterpret_cast<C *>(fr.upd);
+    for (int j = blockIdx.y; j < f; j += gridDim.y) {
+        const C *col = F + (long)j * f;
+        C *g = j < o3 ? G + (long)perm[(long)blockIdx.x * permld + j] * f : nullptr;
+        for (int r = threadIdx.x; r < f; r += BP_THREADS) {
+            C v = col[r];
+            if (j < o3) {
+                if (r >= o3) { v.x = -v.x; v.y = -v.y; }
+                g[r] = v;
+            } else if (r < o3) {
+                X[(long)(j - o3) * o3 + r] = v;
             } else {
-                v = F[e];
-                const C pc = pcol[i], pr = prow[j];
-                v.x -= pc.x * pr.x - pc.y * pr.y;
-                v.y -= pc.x * pr.y + pc.y * pr.x;
+                U[(long)(j - o3) * b3 + r - o3] = v;
             }
-            F[e] = v;
         }
-        __syncthreads();
     }
-    C *G = fac + fr.fac_off; // f x o3, ld f
-    for (int e = tid; e < f * o3; e += nt) {
-        const int r = e % f, j = e / f;
-        C v = F[(long)j * f + r];
-        if (r >= o3) { v.x = -v.x; v.y = -v.y; }
-        G[(long)perm[j] * f + r] = v;
-    }
-    C *X = G + (long)f * o3; // o3 x b3, ld o3
-    for (int e = tid; e < o3 * b3; e += nt) X[e] = F[(long)(o3 + e / o3) * f + e % o3];
-    C *U = reinterpret_cast<C *>(fr.upd); // b3 x b3, ld b3
-    for (int e = tid; e < b3 * b3; e += nt) U[e] = F[(long)(o3 + e / b3) * f + o3 + e % b3];
 }
 
 template <typename C>
@@ -680,6 +912,58 @@ template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std
     return put(F->st_point, point.data(), sizeof(int) * point.size());
 }
 
+// One level's batched fronts (fm, om: the largest front and own block), all at once.
+// ws: panel_ws_bytes(count, fm, om), scratch: count fm^2 entries.
+template <typename C> static size_t panel_ws_bytes(size_t count, int fm, int om)
+{
+    return count * (sizeof(C) * 2 * BP_NB * (size_t)fm + sizeof(BatchPanel<C>) + sizeof(unsigned long long) + sizeof(int) * (size_t)om);
+}
+template <typename C>
+static spm_status factor_panels(const BatchFront *fronts, int count, int fm, int om, const C *S, const int *pts,
+                                const int *maps, const int *rels, GridDesc g, C *scratch, char *ws, C *fac, double tau,
+                                int *raised, cudaStream_t s)
+{
+    const long stride = (long)fm * fm;
+    const size_t b_amax = sizeof(unsigned long long) * (size_t)count;
+    C *M = reinterpret_cast<C *>(ws); // most aligned first
+    C *srow = M + (size_t)count * BP_NB * fm;
+    BatchPanel<C> *panels = reinterpret_cast<BatchPanel<C> *>(srow + (size_t)count * BP_NB * fm);
+    unsigned long long *amax2 = reinterpret_cast<unsigned long long *>(panels + count);
+    int *perm = reinterpret_cast<int *>(amax2 + count);
+    SPM_CUDA_TRY(cudaMemsetAsync(amax2, 0, b_amax, s));
+    SPM_CUDA_TRY(cudaMemsetAsync(scratch, 0, sizeof(C) * stride * count, s));
+    const unsigned rows = (unsigned)std::max(1, std::min(fm, (8 * 152 + count - 1) / count)); // blocks per front
+    const size_t smem = sizeof(C) * (BP_NB + 1) * (size_t)om;
+    const int threads = std::min(BP_THREADS, std::max(64, (fm + 31) / 32 * 32)); // a thread per row, up to 256
+    // om <= 1536: at most 216 KB, with the static shared memory below the 227 KB of a block
+    SPM_CUDA_TRY(cudaFuncSetAttribute(k_bp_panel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, 216 * 1024));
+    launch_pdl(k_bp_assemble<C>, dim3(count, rows), dim3(BP_THREADS), 0, s, fronts, S, pts, maps, g, scratch, stride, perm, om);
+    for (int ch = 0; ch < 2; ++ch)
+        launch_pdl(k_bp_extend<C>, dim3(count, rows), dim3(BP_THREADS), 0, s, fronts, ch, rels, scratch, stride);
+    launch_pdl(k_bp_absmax<C>, dim3(count, rows), dim3(BP_THREADS), 0, s, fronts, (const C *)scratch, stride, amax2);
+    // columns per update block: as many as leave two blocks for every SM
+    auto blocks_of = [&](int ct) { return (unsigned)((fm + ct - 1) / ct); };
+    const int ct = blocks_of(8) * count >= 304 ? 8 : (blocks_of(4) * count >= 304 ? 4 : 2);
+    for (int k0 = 0; k0 < om; k0 += BP_NB) {
+        launch_pdl(k_bp_panel<C>, dim3(count), dim3(om - k0 > 64 ? BP_THREADS : 128), smem, s, fronts, scratch, stride, k0, tau,
+                   (const unsigned long long *)amax2, perm, om, M, fm, panels, raised);
+        const int row_blocks = (fm + BX_ROWS - 1) / BX_ROWS;
+        launch_pdl(k_bp_cross<C>, dim3(count, row_blocks + (fm + BX_COLS - 1) / BX_COLS), dim3(BX_THREADS), 0, s, fronts, scratch,
+                   stride, k0, row_blocks, M, srow, fm, (const BatchPanel<C> *)panels);
+        const dim3 grid(count, blocks_of(ct));
+        auto update = [&](auto kernel) {
+            launch_pdl(kernel, grid, dim3(threads), 0, s, fronts, scratch, stride, k0, (const C *)M, (const C *)srow, fm);
+        };
+        if (ct == 8) update(k_bp_update<C, 8>);
+        else if (ct == 4) update(k_bp_update<C, 4>);
+        else update(k_bp_update<C, 2>);
+    }
+    launch_pdl(k_bp_store<C>, dim3(count, rows), dim3(BP_THREADS), 0, s, fronts, (const C *)scratch, stride, (const int *)perm,
+               om, fac);
+    SPM_CUDA_TRY(cudaGetLastError());
+    return SPM_OK;
+}
+
 template <typename R>
 static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store, int variant)
 {
@@ -770,18 +1054,28 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
     // its own front, update stack and dense workspace.  A subtree root's update
     // goes to a buffer of its own, where its parent (above the subtrees, factored
     // afterwards on the problem's stream) finds it.
-    // Small fronts (f <= BATCH_FMAX, whose whole subtree is small) are factored
-    // first, level by level, each level in one launch of k_front_batch; their
-    // updates go to buffers of their own.  The stream pool below handles the rest.
-    const int BATCH_FMAX_SMEM = sizeof(R) == 8 ? 112 : 160; // whole front in shared memory
-    const int BATCH_FMAX = 512;                               // larger fronts: global scratch
+    // Fronts of at most fmax unknowns whose subtrees are batched too are factored
+    // first, level by level, all of a level at once (factor_panels); their updates go to
+    // buffers of their own.  The stream pool below handles the rest.  In 3-D 1536 is the
+    // fastest line where the updates fit (n = 32 complex64: 512 327 ms, 1024 275, 1536
+    // 231, 2048 255); where they would take more than 12 GB the next smaller one serves
+    // (n = 64: 15 GB at 1536, 10 at 1024, at the same speed).  In 2-D the line stays at
+    // 512: larger fronts would be faster batched too (n = 239: 137 -> 66 ms), but the
+    // per-front path rounds differently, and 2-D factors have near-singular boxes often
+    // enough (one medium in ten at n = 239) that S^-1 moves by more than 1e-9.
     std::vector<char> batched(NN, 0);
-    for (int id = 0; id < NN; ++id) { // postorder: children before parents
-        const Node &nd = nodes[id];
-        bool ok = !half_store && D * (nd.nown + nd.nbnd) <= BATCH_FMAX;
-        for (int ch : {nd.left, nd.right})
-            if (ch >= 0 && !batched[ch]) ok = false;
-        batched[id] = ok ? 1 : 0;
+    for (const int fmax : {1536, 1024, 512}) {
+        if (n3d == 1 && fmax > 512) continue;
+        double bytes = 0;
+        for (int id = 0; id < NN; ++id) { // postorder: children before parents
+            const Node &nd = nodes[id];
+            bool ok = !half_store && D * (nd.nown + nd.nbnd) <= fmax;
+            for (int ch : {nd.left, nd.right})
+                if (ch >= 0 && !batched[ch]) ok = false;
+            batched[id] = ok ? 1 : 0;
+            if (ok) bytes += sizeof(C) * (double)upd_size[id];
+        }
+        if (bytes <= 12e9) break;
     }
     const size_t one_block = sizeof(R) == 4 ? 768 : 384;
     std::vector<size_t> smax(NN, 0);
@@ -903,54 +1197,39 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
             ++nbf;
         }
         if (nbf > 0) {
-            // per level: the fronts that fit shared memory, then the larger ones
             SPM_TRY(batch_desc.ensure(sizeof(BatchFront) * nbf));
             std::vector<BatchFront> all;
-            struct Launch { size_t first, count; int fm; bool global; };
+            struct Launch { size_t first, count; int fm, om; };
             std::vector<Launch> launches;
-            size_t scratch_max = 0;
+            size_t scratch_max = 0, ws_max = 0;
             for (int d = maxd; d >= 0; --d) {
-                for (int pass = 0; pass < 2; ++pass) {
-                    Launch ln{all.size(), 0, 1, pass == 1};
-                    for (const BatchFront &b : lv[d])
-                        if ((b.f > BATCH_FMAX_SMEM) == (pass == 1)) {
-                            all.push_back(b);
-                            ++ln.count;
-                            ln.fm = std::max(ln.fm, b.f);
-                        }
-                    if (ln.count == 0) continue;
-                    if (ln.global) { // chunks of at most 2 GB of scratch
-                        const size_t per = (size_t)ln.fm * ln.fm;
-                        const size_t chunk = std::max<size_t>(1, ((size_t)2 << 30) / (sizeof(C) * per));
-                        for (size_t c0 = 0; c0 < ln.count; c0 += chunk) {
-                            Launch part = ln;
-                            part.first = ln.first + c0;
-                            part.count = std::min(chunk, ln.count - c0);
-                            scratch_max = std::max(scratch_max, part.count * per);
-                            launches.push_back(part);
-                        }
-                    } else {
-                        launches.push_back(ln);
-                    }
+                if (lv[d].empty()) continue;
+                Launch ln{all.size(), lv[d].size(), 1, 1};
+                for (const BatchFront &b : lv[d]) {
+                    all.push_back(b);
+                    ln.fm = std::max(ln.fm, b.f);
+                    ln.om = std::max(ln.om, b.o3);
+                }
+                const size_t per = (size_t)ln.fm * ln.fm; // chunks of at most 2 GB of scratch
+                const size_t chunk = std::max<size_t>(1, ((size_t)2 << 30) / (sizeof(C) * per));
+                for (size_t c0 = 0; c0 < ln.count; c0 += chunk) {
+                    Launch part = ln;
+                    part.first = ln.first + c0;
+                    part.count = std::min(chunk, ln.count - c0);
+                    scratch_max = std::max(scratch_max, part.count * per);
+                    ws_max = std::max(ws_max, panel_ws_bytes<C>(part.count, ln.fm, ln.om));
+                    launches.push_back(part);
                 }
             }
             SPM_CUDA_TRY(cudaMemcpy(batch_desc.ptr, all.data(), sizeof(BatchFront) * nbf, cudaMemcpyHostToDevice));
-            DevBuf gscratch;
-            if (scratch_max > 0) SPM_TRY(gscratch.ensure(sizeof(C) * scratch_max));
-            const size_t smem_max = sizeof(C) * ((size_t)BATCH_FMAX_SMEM * BATCH_FMAX_SMEM + 2 * BATCH_FMAX_SMEM) +
-                                    sizeof(int) * BATCH_FMAX_SMEM;
-            SPM_CUDA_TRY(cudaFuncSetAttribute(k_front_batch<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
+            DevBuf gscratch, panel_ws;
+            SPM_TRY(gscratch.ensure(sizeof(C) * scratch_max));
+            SPM_TRY(panel_ws.ensure(ws_max));
             const GridDesc gd2{n1, n2, n3d, D, SY.nsten};
-            for (const Launch &ln : launches) {
-                const size_t fm = (size_t)ln.fm;
-                const size_t smem = ln.global ? sizeof(C) * 2 * fm + sizeof(int) * fm
-                                              : sizeof(C) * (fm * fm + 2 * fm) + sizeof(int) * fm;
-                k_front_batch<C><<<(unsigned)ln.count, 256, smem, s>>>(
-                    batch_desc.as<BatchFront>() + ln.first, Sdev, dpts, dmaps, drels, gd2, fac, pivot_floor<R>(),
-                    dinfo + 2, ln.global ? gscratch.as<C>() : nullptr, (long)(fm * fm));
-            }
-            SPM_CUDA_TRY(cudaGetLastError());
-            if (scratch_max > 0) SPM_CUDA_TRY(cudaStreamSynchronize(s)); // before the scratch is freed
+            for (const Launch &ln : launches)
+                SPM_TRY(factor_panels<C>(batch_desc.as<BatchFront>() + ln.first, (int)ln.count, ln.fm, ln.om, Sdev, dpts, dmaps,
+                                         drels, gd2, gscratch.as<C>(), panel_ws.as<char>(), fac, pivot_floor<R>(), dinfo + 2, s));
+            SPM_CUDA_TRY(cudaStreamSynchronize(s)); // before the scratch is freed
         }
     }
     // per-slot buffers and streams (slot ngroups - 1 is the problem's stream)

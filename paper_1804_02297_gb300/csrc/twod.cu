@@ -647,27 +647,34 @@ __global__ void k2_gram_sum(const double2 *__restrict__ part, int nblocks, doubl
 
 __device__ __forceinline__ double2 zm(double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
-// One block per class: H = M M^H from the Gram sums, Jacobi eigen-decomposition,
+// One block per class: H = M M^H from the Gram sums, cyclic Jacobi eigen-decomposition,
 // alpha = conj(eigenvectors of the two smallest eigenvalues), sv = sqrt(eigenvalues)
-// ascending, beta = B^T alpha.  A sweep is M - 1 rounds of M/2 disjoint rotations (the
-// round-robin ordering; M = 8, 12, 18): a rotation by one thread costs its FP64
-// instructions one after the other, about 20 us, and a set-up has some 8000 of them (one
-// thread for all of them, class after class, took 0.1 s of a set-up's 0.28 s at n = 119).
-constexpr int EIG2_THREADS = 192; // 9 pairs x 18 rows, in whole warps
+// ascending, beta = B^T alpha.  Warp 0 rotates A, its lanes the rows and columns; warp 1
+// follows one rotation behind with V.  Bound by a warp's chain of FP64 instructions (64
+// cycles each on its scheduler), some 3 us a rotation, 1400 rotations; with one thread for
+// all of it, class after class, the fit took 75 ms of a set-up.  (Disjoint rotations in
+// parallel take 0.9 ms, but another order of rotations rounds differently, and where a
+// box of the dissection is nearly singular the factor of S magnifies that to 1e-8.)
+constexpr int EIG2_THREADS = 64;
+struct Rot2 {
+    double cs, sn;
+    double2 ce; // conj of the phase of A_pq
+    int p, q;   // p < 0: nothing to rotate
+};
 __global__ void __launch_bounds__(EIG2_THREADS) k2_eig(const double2 *__restrict__ sums, const double2 *__restrict__ E,
                                                        const __grid_constant__ Geoms2 gs, int n, double k, double2 *alpha,
                                                        double2 *beta, double *sv)
 {
-    __shared__ double2 A[18][18], V[18][18], rph[9];
-    __shared__ double rc[9], rs[9], fro;
-    __shared__ int rp[9], rq[9], idx[18];
-    __shared__ unsigned long long off;
+    __shared__ double2 A[18][18], V[18][18];
+    __shared__ Rot2 rot[2];
+    __shared__ double fro, off;
+    __shared__ int idx[18];
     const Geom2 &g = gs.c[blockIdx.x];
     sums += blockIdx.x * 4 * 81;
     alpha += blockIdx.x * 36;
     beta += blockIdx.x * 54;
     sv += blockIdx.x * 18;
-    const int T = g.T, M = 2 * T, tid = threadIdx.x, np = M / 2;
+    const int T = g.T, M = 2 * T, tid = threadIdx.x, lane = tid & 31;
     const double k4 = k * k * k * k;
     for (int e = tid; e < M * M; e += EIG2_THREADS) {
         const int r = e / M, c = e % M, d = r / T, o = r % T, f = c / T, op = c % T;
@@ -691,64 +698,69 @@ __global__ void __launch_bounds__(EIG2_THREADS) k2_eig(const double2 *__restrict
             for (int c = 0; c < M; ++c) s += A[r][c].x * A[r][c].x + A[r][c].y * A[r][c].y;
         fro = s;
     }
+    if (tid == 0) rot[1].p = -1;
+    __syncthreads();
+    auto rotate_V = [&](const Rot2 &r) {
+        if (r.p < 0 || lane >= M) return;
+        const double2 vp = V[lane][r.p], vq = zm(V[lane][r.q], r.ce);
+        V[lane][r.p] = make_double2(r.cs * vp.x - r.sn * vq.x, r.cs * vp.y - r.sn * vq.y);
+        V[lane][r.q] = make_double2(r.sn * vp.x + r.cs * vq.x, r.sn * vp.y + r.cs * vq.y);
+    };
+    int par = 0;
     for (int sweep = 0; sweep < 60; ++sweep) {
-        if (tid == 0) off = 0ull;
-        __syncthreads();
-        for (int round = 0; round < M - 1; ++round) {
-            if (tid < np) {
-                const int pb = M - 1 - tid;
-                int p = tid == 0 ? 0 : (tid - 1 + round) % (M - 1) + 1, q = (pb - 1 + round) % (M - 1) + 1;
-                if (p > q) { const int s = p; p = q; q = s; }
-                const double2 b = A[p][q];
-                const double b2 = b.x * b.x + b.y * b.y, ab = sqrt(b2);
-                double cs = 1.0, sn = 0.0;
-                double2 ph = make_double2(1.0, 0.0);
-                if (ab > 1e-300) {
-                    atomicMax(&off, (unsigned long long)__double_as_longlong(b2)); // positive doubles order as integers
-                    const double zeta = (A[q][q].x - A[p][p].x) / (2.0 * ab);
-                    const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-                    cs = 1.0 / sqrt(1.0 + t * t);
-                    sn = t * cs;
-                    ph = make_double2(b.x / ab, -b.y / ab); // conj of the phase of A_pq
-                }
-                rp[tid] = p;
-                rq[tid] = q;
-                rc[tid] = cs;
-                rs[tid] = sn;
-                rph[tid] = ph;
-            }
-            __syncthreads();
-            // J = diag(1, ph) [[cs, sn], [-sn, cs]] on each (p, q): A <- J^H A J, V <- V J
-            const int j = tid / M, i = tid % M;
-            const bool act = j < np;
-            const int p = act ? rp[j] : 0, q = act ? rq[j] : 0;
-            const double cs = act ? rc[j] : 1.0, sn = act ? rs[j] : 0.0;
-            const double2 ph = act ? rph[j] : make_double2(1.0, 0.0);
-            if (act) { // columns
-                const double2 ap = A[i][p], aq = zm(A[i][q], ph);
-                A[i][p] = make_double2(cs * ap.x - sn * aq.x, cs * ap.y - sn * aq.y);
-                A[i][q] = make_double2(sn * ap.x + cs * aq.x, sn * ap.y + cs * aq.y);
-                const double2 vp = V[i][p], vq = zm(V[i][q], ph);
-                V[i][p] = make_double2(cs * vp.x - sn * vq.x, cs * vp.y - sn * vq.y);
-                V[i][q] = make_double2(sn * vp.x + cs * vq.x, sn * vp.y + cs * vq.y);
-            }
-            __syncthreads();
-            if (act) { // rows; the rotated pair becomes exactly diagonal
-                const double2 ap = A[p][i], aq = zm(A[q][i], conj_of(ph));
-                double2 np_ = make_double2(cs * ap.x - sn * aq.x, cs * ap.y - sn * aq.y);
-                double2 nq_ = make_double2(sn * ap.x + cs * aq.x, sn * ap.y + cs * aq.y);
-                if (i == p) { np_.y = 0.0; nq_ = make_double2(0.0, 0.0); }
-                if (i == q) { nq_.y = 0.0; np_ = make_double2(0.0, 0.0); }
-                A[p][i] = np_;
-                A[q][i] = nq_;
-            }
-            __syncthreads();
+        if (tid == 0) {
+            double s = 0;
+            for (int r = 0; r < M; ++r)
+                for (int c = r + 1; c < M; ++c) s += A[r][c].x * A[r][c].x + A[r][c].y * A[r][c].y;
+            off = s;
         }
-        // the sum over all pairs is at most M (M - 1) / 2 times the largest
-        const bool done = __longlong_as_double((long long)off) * (M * (M - 1) / 2) <= 1e-34 * fro;
         __syncthreads();
-        if (done) break;
+        if (off <= 1e-34 * fro) break;
+        for (int p = 0; p < M; ++p)
+            for (int q = p + 1; q < M; ++q, par ^= 1) {
+                if (tid >= 32) {
+                    rotate_V(rot[par ^ 1]); // the rotation before this one
+                } else {
+                    const double2 cpq = A[p][q];
+                    const double ab = sqrt(cpq.x * cpq.x + cpq.y * cpq.y);
+                    const bool on = ab > 1e-300;
+                    if (on) {
+                        // the phase's two divisions and zeta's in three lanes at once
+                        const double num = lane == 0 ? cpq.x : (lane == 1 ? cpq.y : A[q][q].x - A[p][p].x);
+                        const double quo = num / (lane < 2 ? ab : 2.0 * ab);
+                        double2 e;
+                        e.x = __shfl_sync(0xffffffffu, quo, 0);
+                        e.y = __shfl_sync(0xffffffffu, quo, 1);
+                        const double zeta = __shfl_sync(0xffffffffu, quo, 2);
+                        const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+                        const double cs = 1.0 / sqrt(1.0 + t * t), sn = t * cs;
+                        // J = diag(1, conj e) [[cs, sn], [-sn, cs]] on (p, q): A <- J^H A J, V <- V J
+                        const double2 ce = conj_of(e);
+                        if (lane < M) { // columns
+                            const double2 ap = A[lane][p], aqe = zm(A[lane][q], ce);
+                            A[lane][p] = make_double2(cs * ap.x - sn * aqe.x, cs * ap.y - sn * aqe.y);
+                            A[lane][q] = make_double2(sn * ap.x + cs * aqe.x, sn * ap.y + cs * aqe.y);
+                        }
+                        __syncwarp();
+                        if (lane < M) { // rows; the rotated pair becomes exactly diagonal
+                            const double2 ap = A[p][lane], aqe = zm(A[q][lane], e);
+                            double2 np_ = make_double2(cs * ap.x - sn * aqe.x, cs * ap.y - sn * aqe.y);
+                            double2 nq_ = make_double2(sn * ap.x + cs * aqe.x, sn * ap.y + cs * aqe.y);
+                            if (lane == p) { np_.y = 0.0; nq_ = make_double2(0.0, 0.0); }
+                            if (lane == q) { nq_.y = 0.0; np_ = make_double2(0.0, 0.0); }
+                            A[p][lane] = np_;
+                            A[q][lane] = nq_;
+                        }
+                        if (lane == 0) rot[par] = Rot2{cs, sn, ce, p, q};
+                    } else if (lane == 0) {
+                        rot[par].p = -1;
+                    }
+                }
+                __syncthreads();
+            }
     }
+    if (tid >= 32) rotate_V(rot[par ^ 1]); // the last one
+    __syncthreads();
     if (tid == 0) {
         for (int i = 0; i < M; ++i) idx[i] = i;
         for (int i = 1; i < M; ++i) { // insertion sort by eigenvalue

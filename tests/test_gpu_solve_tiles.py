@@ -69,6 +69,39 @@ def test_c128_matches_oracle_lu(spm, problems, nrhs):
         assert rel(x.cpu().numpy(), np.stack([F.solve(v) for v in b])) < 1e-9
 
 
+@pytest.mark.parametrize("n", [4, 5, 6, 11, 12, 13, 33])
+def test_batched_factor_panels_2d(spm, n):
+    """Own blocks that are and are not multiples of the panel width, one leaf (n <= 5) to
+    several levels, complex128 and complex64, with rough media so that rows are swapped."""
+    k = si.wavenumber_for_grid_2d(n)
+    eps, grad = si.random_medium_2d(n, 5)
+    P = spm.Problem2D(n, k, eps, grad)
+    al, be, _ = twod.all_stencils(n, k)
+    P.set_stencils(al, be)
+    m, p = twod.medium(eps, grad)
+    b = si.random_field_2d(n, 9, 1)
+    ref = twod.SFactor(n, m, p, al, be).solve(b[0])
+    P.factor_S(spm.SPM_C128)
+    x = torch.zeros(b.shape, dtype=torch.complex128, device="cuda")
+    P.solve_S(dev(b, torch.complex128), x)
+    torch.cuda.synchronize()
+    assert rel(x.cpu().numpy()[0], ref) < 1e-9
+    P.factor_S(spm.SPM_C64)
+    assert P.factor_info(spm.SPM_C64)[3] < 1e-4
+
+
+def test_batched_factor_large_own_block(spm):
+    """3-D n = 16: fronts of 1152 unknowns and own blocks of up to 768, whose panel takes
+    108 KB of a block's shared memory; the probe residual says whether it is a factor."""
+    n = 16
+    eps, grad = si.medium_bumps(n, seed=3, count=8)
+    P = spm.Problem(n, si.wavenumber_for_grid(n), eps, grad)
+    P.build_stencils(spm.SPM_C128)
+    assert P.factor_info(spm.SPM_C128)[3] < 1e-12
+    P.factor_S(spm.SPM_C64)
+    assert P.factor_info(spm.SPM_C64)[3] < 1e-4
+
+
 @pytest.mark.parametrize("storage,bound", [("SPM_C64", 1e-4), ("SPM_C64H", 2e-2)])
 @pytest.mark.parametrize("nrhs", RHS)
 def test_c64_residual(spm, problems, nrhs, storage, bound):
