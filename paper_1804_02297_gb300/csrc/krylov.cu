@@ -1,6 +1,7 @@
 // Incident fields, BLAS-1 helpers and the preconditioned GMRES driver.
 #include <math.h>
 
+#include <algorithm>
 #include <complex>
 #include <vector>
 
@@ -85,35 +86,47 @@ spm_status spm_axpby_impl(int prec, long count, double a, const void *x, double 
 // operator and preconditioner application acts on the whole batch.
 namespace {
 
-constexpr int DOT_BLOCKS = 304; // 2 x 152 SMs
-constexpr int VGROUP = 8;       // basis vectors per dot/axpy pass
+// Reductions over a vector.  FP64 arithmetic on two lanes per SM is what they cost, the
+// sums across a warp included (a shuffled FP64 sum of eight products is 80 additions, 64
+// cycles each on the warp's scheduler), so a block is four warps, one per scheduler, with
+// as many elements per thread as that leaves.  Each block stores its partial sums; the
+// last one to finish adds them up, in block order.  At n = 32 and one right-hand side a
+// pass over five vectors took 30 us plus 50 us for the separate launch whose eight threads
+// added 304 partial sums each; now 12 us.
+constexpr int DOT_BLOCKS = 304, DOT_THREADS = 128;
+constexpr int VGROUP = 8; // basis vectors per dot/axpy pass
 
-// partial[b][blk][i] = sum over this block's k of conj(V_i[b][k]) w[b][k]
-template <typename C>
-__global__ void k_dots(const C *__restrict__ V, long vstride, int i0, int ni, const C *__restrict__ w, long N,
-                       int nrhs, double2 *__restrict__ partial)
+// float -> double by integer arithmetic (exponent rebiased, 29 zero bits appended): the
+// conversion instruction goes through the FP64 pipe, which is what these kernels wait for.
+// Zeros, subnormals, infinities and NaNs take the instruction.
+__device__ __forceinline__ double widen(float a)
 {
-    __shared__ double2 red[VGROUP][8];
-    const int b = blockIdx.y;
-    double2 acc[VGROUP];
+    const unsigned b = __float_as_uint(a), e = (b >> 23) & 255u;
+    if (e - 1u >= 254u) return (double)a;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+__device__ __forceinline__ double widen(double a) { return a; }
+
+inline int dot_blocks(long N, int nrhs)
+{
+    const long most = std::max(16, DOT_BLOCKS / nrhs); // blocks per right-hand side
+    return (int)std::max(1L, std::min({(long)DOT_BLOCKS / 2, most, (N + DOT_THREADS - 1) / DOT_THREADS}));
+}
+
+// The block's sums of acc[0 .. NV) over its threads go to partial[b][blk][i]; true in the
+// last block of right-hand side b to get here, whose total[i] then holds the sums over
+// all blocks (shared memory, visible to every thread).  done: a zeroed counter per
+// right-hand side, zeroed again on the way out.
+template <int NV>
+__device__ bool reduce_last(const double2 (&acc)[NV], int nv, double2 *__restrict__ partial, int b, unsigned *done,
+                            double2 *total)
+{
+    __shared__ double2 red[NV][DOT_THREADS / 32];
+    __shared__ bool last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nblk = gridDim.x;
 #pragma unroll
-    for (int i = 0; i < VGROUP; ++i) acc[i] = make_double2(0, 0);
-    const C *wb = w + (long)b * N;
-    for (long k = (long)blockIdx.x * blockDim.x + threadIdx.x; k < N; k += (long)gridDim.x * blockDim.x) {
-        C wk = wb[k];
-        double wx = wk.x, wy = wk.y;
-#pragma unroll
-        for (int i = 0; i < VGROUP; ++i) {
-            if (i < ni) {
-                C v = V[(long)(i0 + i) * vstride + (long)b * N + k];
-                acc[i].x += (double)v.x * wx + (double)v.y * wy;
-                acc[i].y += (double)v.x * wy - (double)v.y * wx;
-            }
-        }
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < VGROUP; ++i) {
+    for (int i = 0; i < NV; ++i) {
+        if (i >= nv) break;
         double x = acc[i].x, y = acc[i].y;
         for (int off = 16; off > 0; off >>= 1) {
             x += __shfl_down_sync(0xffffffffu, x, off);
@@ -122,45 +135,105 @@ __global__ void k_dots(const C *__restrict__ V, long vstride, int i0, int ni, co
         if (lane == 0) red[i][wid] = make_double2(x, y);
     }
     __syncthreads();
-    if (threadIdx.x < ni) {
-        double2 s = make_double2(0, 0);
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) { s.x += red[threadIdx.x][q].x; s.y += red[threadIdx.x][q].y; }
-        partial[((long)b * gridDim.x + blockIdx.x) * VGROUP + threadIdx.x] = s;
+    double2 *pb = partial + (long)b * nblk * VGROUP;
+    if (threadIdx.x < nv) {
+        double2 s = red[threadIdx.x][0];
+        for (int q = 1; q < DOT_THREADS / 32; ++q) { s.x += red[threadIdx.x][q].x; s.y += red[threadIdx.x][q].y; }
+        pb[(long)blockIdx.x * VGROUP + threadIdx.x] = s;
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&done[b], 1u) == (unsigned)nblk - 1;
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+    for (int i = wid; i < nv; i += DOT_THREADS / 32) { // a warp per sum
+        double x = 0, y = 0;
+        for (int q = lane; q < nblk; q += 32) {
+            const double2 v = __ldcg(&pb[(long)q * VGROUP + i]);
+            x += v.x;
+            y += v.y;
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            x += __shfl_down_sync(0xffffffffu, x, off);
+            y += __shfl_down_sync(0xffffffffu, y, off);
+        }
+        if (lane == 0) total[i] = make_double2(x, y);
+    }
+    if (threadIdx.x == 0) done[b] = 0;
+    __syncthreads();
+    return true;
 }
 
-// out[b][i] = sum over blocks of partial[b][blk][i]
-__global__ void k_dots_finish(const double2 *__restrict__ partial, int nblk, int ni, int nrhs, double2 *out, int ld,
-                              int i0)
+// out[b][i0 + i] = <V_{i0+i}[b], w[b]>, i < ni
+template <typename C>
+__global__ void __launch_bounds__(DOT_THREADS) k_dots(const C *__restrict__ V, long vstride, int i0, int ni,
+                                                      const C *__restrict__ w, long N, double2 *__restrict__ partial,
+                                                      unsigned *done, double2 *out, int ld)
 {
-    int b = blockIdx.x, i = threadIdx.x;
-    if (i >= ni) return;
-    double2 s = make_double2(0, 0);
-    for (int q = 0; q < nblk; ++q) {
-        double2 v = partial[((long)b * nblk + q) * VGROUP + i];
-        s.x += v.x;
-        s.y += v.y;
+    pdl_wait_and_trigger();
+    __shared__ double2 total[VGROUP];
+    const int b = blockIdx.y;
+    double2 acc[VGROUP];
+#pragma unroll
+    for (int i = 0; i < VGROUP; ++i) acc[i] = make_double2(0, 0);
+    const C *wb = w + (long)b * N, *vb = V + (long)i0 * vstride + (long)b * N;
+    for (long k = (long)blockIdx.x * DOT_THREADS + threadIdx.x; k < N; k += (long)gridDim.x * DOT_THREADS) {
+        const C wk = wb[k];
+        const double wx = widen(wk.x), wy = widen(wk.y);
+#pragma unroll
+        for (int i = 0; i < VGROUP; ++i) {
+            if (i < ni) {
+                const C v = vb[(long)i * vstride + k];
+                const double vx = widen(v.x), vy = widen(v.y);
+                acc[i].x = fma(vx, wx, fma(vy, wy, acc[i].x));
+                acc[i].y = fma(vx, wy, fma(-vy, wx, acc[i].y));
+            }
+        }
     }
-    out[(long)b * ld + i0 + i] = s;
+    if (reduce_last(acc, ni, partial, b, done, total) && threadIdx.x < ni) out[(long)b * ld + i0 + threadIdx.x] = total[threadIdx.x];
 }
 
-// w[b] -= sum_{i < ni} h[b][i0+i] V_{i0+i}[b]   (coefficients FP64)
+// r = g - Ax, out[b] = ||r[b]||^2
+__global__ void __launch_bounds__(DOT_THREADS) k_residual(double2 *r, const double2 *__restrict__ g, const double2 *__restrict__ Ax,
+                                                          long N, double2 *__restrict__ partial, unsigned *done, double2 *out,
+                                                          int ld)
+{
+    pdl_wait_and_trigger();
+    __shared__ double2 total[1];
+    const long b = blockIdx.y;
+    double2 acc[1] = {make_double2(0, 0)};
+    for (long k = (long)blockIdx.x * DOT_THREADS + threadIdx.x; k < N; k += (long)gridDim.x * DOT_THREADS) {
+        double2 v = g[b * N + k];
+        const double2 a = Ax[b * N + k];
+        v.x -= a.x;
+        v.y -= a.y;
+        r[b * N + k] = v;
+        acc[0].x = fma(v.x, v.x, fma(v.y, v.y, acc[0].x));
+    }
+    if (reduce_last(acc, 1, partial, (int)b, done, total) && threadIdx.x == 0) out[b * ld] = total[0];
+}
+
+// w[b] += sign sum_{i < ni} h[b][i0+i] V_{i0+i}[b], sign = +-1   (coefficients FP64)
 template <typename C>
 __global__ void k_axpy_multi(const C *__restrict__ V, long vstride, int i0, int ni, const double2 *__restrict__ h,
                              int ld, C *w, long N, int nrhs, double sign)
 {
     long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait_and_trigger();
     if (gid >= N * nrhs) return;
-    long b = gid / N, k = gid - b * N;
+    const long b = gid / N;
     C wk = w[gid];
-    double x = wk.x, y = wk.y;
-    for (int i = 0; i < ni; ++i) {
-        double2 c = h[b * ld + i0 + i];
-        C v = V[(long)(i0 + i) * vstride + gid];
-        x += sign * (c.x * v.x - c.y * v.y);
-        y += sign * (c.x * v.y + c.y * v.x);
+    double x = widen(wk.x), y = widen(wk.y);
+#pragma unroll
+    for (int i = 0; i < VGROUP; ++i) {
+        if (i >= ni) break;
+        const double2 c = h[b * ld + i0 + i];
+        const C v = V[(long)(i0 + i) * vstride + gid];
+        const double vx = widen(v.x), vy = widen(v.y), cx = sign < 0 ? -c.x : c.x, cy = sign < 0 ? -c.y : c.y;
+        x = fma(cx, vx, fma(-cy, vy, x));
+        y = fma(cx, vy, fma(cy, vx, y));
     }
-    (void)k;
     wk.x = x;
     wk.y = y;
     w[gid] = wk;
@@ -171,6 +244,7 @@ template <typename C, typename D>
 __global__ void k_scale_copy(D *dst, const C *__restrict__ src, const double *__restrict__ scale, long N, int nrhs)
 {
     long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait_and_trigger();
     if (gid >= N * nrhs) return;
     double s = scale[gid / N];
     C v = src[gid];
@@ -185,6 +259,7 @@ template <typename C>
 __global__ void k_accum(double2 *x, const C *__restrict__ d, const double *__restrict__ scale, long N, int nrhs)
 {
     long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait_and_trigger();
     if (gid >= N * nrhs) return;
     double s = scale[gid / N];
     C v = d[gid];
@@ -196,14 +271,20 @@ __global__ void k_accum(double2 *x, const C *__restrict__ d, const double *__res
 
 inline unsigned nblocks(long cnt) { return (unsigned)((cnt + 255) / 256); }
 
+// where the reductions keep their partial sums and count their finished blocks
+struct Reduce {
+    double2 *partial; // [nrhs][DOT_BLOCKS][VGROUP]
+    unsigned *done;   // [nrhs], zero between launches
+};
+
 template <typename C>
-spm_status dots(const C *V, long vstride, int nvec, const C *w, long N, int nrhs, double2 *partial, double2 *out,
-                int ld, cudaStream_t s)
+spm_status dots(const C *V, long vstride, int nvec, const C *w, long N, int nrhs, const Reduce &rd, double2 *out, int ld,
+                cudaStream_t s)
 {
     for (int i0 = 0; i0 < nvec; i0 += VGROUP) {
         int ni = nvec - i0 < VGROUP ? nvec - i0 : VGROUP;
-        k_dots<C><<<dim3(DOT_BLOCKS, nrhs), 256, 0, s>>>(V, vstride, i0, ni, w, N, nrhs, partial);
-        k_dots_finish<<<nrhs, VGROUP, 0, s>>>(partial, DOT_BLOCKS, ni, nrhs, out, ld, i0);
+        launch_pdl(k_dots<C>, dim3(dot_blocks(N, nrhs), nrhs), dim3(DOT_THREADS), 0, s, V, vstride, i0, ni, w, N, rd.partial,
+                   rd.done, out, ld);
     }
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
@@ -215,7 +296,7 @@ spm_status axpy_multi(const C *V, long vstride, int nvec, const double2 *h, int 
 {
     for (int i0 = 0; i0 < nvec; i0 += VGROUP) {
         int ni = nvec - i0 < VGROUP ? nvec - i0 : VGROUP;
-        k_axpy_multi<C><<<nblocks(N * nrhs), 256, 0, s>>>(V, vstride, i0, ni, h, ld, w, N, nrhs, sign);
+        launch_pdl(k_axpy_multi<C>, dim3(nblocks(N * nrhs)), dim3(256), 0, s, V, vstride, i0, ni, h, ld, w, N, nrhs, sign);
     }
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
@@ -251,20 +332,18 @@ __device__ __forceinline__ double2 zmul(double2 a, double2 b) { return make_doub
 __device__ __forceinline__ double2 zconj(double2 a) { return make_double2(a.x, -a.y); }
 __device__ __forceinline__ double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
-// Arnoldi step j: column j of H from the two Gram-Schmidt passes (h1, h2) and
-// ||w|| (nn), the previous rotations applied, a new rotation that zeroes
+// Arnoldi step j of right-hand side b: column j of H from the two Gram-Schmidt passes
+// (h1, h2) and ||w||^2, the previous rotations applied, a new rotation that zeroes
 // H[j+1][j], g rotated; scale = 1/||w|| for normalising v_{j+1}; a RHS whose
 // |g[j+1]| <= rtol beta (or whose ||w|| vanished) becomes inactive.
-__global__ void k_arnoldi_givens(GmresSmall gs, const double2 *__restrict__ h1, const double2 *__restrict__ h2,
-                                 const double2 *__restrict__ nn, int ld, int j, int restart, int nrhs)
+__device__ void arnoldi_givens(const GmresSmall &gs, const double2 *h1, const double2 *h2, double nn, int ld, int j, int restart,
+                               int b)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nrhs) return;
     if (!gs.active[b]) { gs.scale[b] = 0.0; return; }
     double2 *H = gs.H + (long)b * (restart + 1) * restart;
     double2 *cs = gs.cs + (long)b * restart, *sn = gs.sn + (long)b * restart, *g = gs.g + (long)b * (restart + 1);
     for (int i = 0; i <= j; ++i) H[i * restart + j] = zadd(h1[(long)b * ld + i], h2[(long)b * ld + i]);
-    const double hn = sqrt(fmax(nn[(long)b * ld].x, 0.0));
+    const double hn = sqrt(fmax(nn, 0.0));
     if (!isfinite(hn)) { atomicAdd(&gs.count[1], 1); gs.active[b] = 0; gs.scale[b] = 0.0; return; }
     H[(j + 1) * restart + j] = make_double2(hn, 0.0);
     gs.scale[b] = hn > 1e-300 ? 1.0 / hn : 0.0;
@@ -287,6 +366,46 @@ __global__ void k_arnoldi_givens(GmresSmall gs, const double2 *__restrict__ h1, 
     const double r = sqrt(g[j + 1].x * g[j + 1].x + g[j + 1].y * g[j + 1].y);
     if (r <= gs.rtol[b] * gs.beta[b] || hn <= 1e-300) gs.active[b] = 0;
     else atomicAdd(&gs.count[0], 1);
+}
+
+// The end of Arnoldi step j in one launch: w[b] -= sum_{i < ni} h2[b][i0+i] V_{i0+i}[b] (the
+// last group of the second Gram-Schmidt pass), ||w||^2 and the small problem's step, by the
+// last block of each right-hand side.
+template <typename C>
+__global__ void __launch_bounds__(DOT_THREADS) k_arnoldi_end(const C *__restrict__ V, long vstride, int i0, int ni, const double2 *h1,
+                                                             const double2 *h2, int ld, C *w, long N,
+                                                             double2 *__restrict__ partial, unsigned *done, GmresSmall gs,
+                                                             int j, int restart)
+{
+    pdl_wait_and_trigger();
+    __shared__ double2 total[1], h[VGROUP];
+    const int b = blockIdx.y;
+    if (threadIdx.x < ni) h[threadIdx.x] = h2[(long)b * ld + i0 + threadIdx.x];
+    __syncthreads();
+    double2 acc[1] = {make_double2(0, 0)};
+    C *wb = w + (long)b * N;
+    const C *vb = V + (long)i0 * vstride + (long)b * N;
+    for (long k = (long)blockIdx.x * DOT_THREADS + threadIdx.x; k < N; k += (long)gridDim.x * DOT_THREADS) {
+        C wk = wb[k];
+        double x = widen(wk.x), y = widen(wk.y);
+#pragma unroll
+        for (int i = 0; i < VGROUP; ++i) {
+            if (i < ni) {
+                const C v = vb[(long)i * vstride + k];
+                const double vx = widen(v.x), vy = widen(v.y);
+                x = fma(-h[i].x, vx, fma(h[i].y, vy, x));
+                y = fma(-h[i].x, vy, fma(-h[i].y, vx, y));
+            }
+        }
+        wk.x = x;
+        wk.y = y;
+        wb[k] = wk;
+        x = widen(wk.x);
+        y = widen(wk.y);
+        acc[0].x = fma(x, x, fma(y, y, acc[0].x));
+    }
+    if (reduce_last(acc, 1, partial, b, done, total) && threadIdx.x == 0)
+        arnoldi_givens(gs, h1, h2, total[0].x, ld, j, restart, b);
 }
 
 // back substitution H y = g over the leading m columns (fewer where a RHS
@@ -319,7 +438,7 @@ __global__ void k_backsolve(GmresSmall gs, double2 *coef, int ld, int m, int res
 template <typename R>
 spm_status gmres_cycle(const KrylovOps &ops, int prec, const typename cplx_of<R>::type *r,
                        typename cplx_of<R>::type *d, int nrhs, int restart, typename cplx_of<R>::type *V,
-                       typename cplx_of<R>::type *tmp, double2 *partial, double2 *h1, double2 *h2, double2 *nn,
+                       typename cplx_of<R>::type *tmp, const Reduce &rd, double2 *h1, double2 *h2, double2 *nn,
                        const GmresSmall &gs, int *count_host, int *iters, cudaStream_t s)
 {
     using C = typename cplx_of<R>::type;
@@ -332,7 +451,7 @@ spm_status gmres_cycle(const KrylovOps &ops, int prec, const typename cplx_of<R>
     // v0 = S^{-1} Q r / beta
     SPM_TRY(ops.apply_Q(ops.ctx, prec, r, tmp, nrhs, s));
     SPM_TRY(ops.solve_S(ops.ctx, prec, tmp, V, nrhs, s));
-    SPM_TRY(dots<C>(V, vstride, 1, V, N, nrhs, partial, nn, ld, s));
+    SPM_TRY(dots<C>(V, vstride, 1, V, N, nrhs, rd, nn, ld, s));
     SPM_CUDA_TRY(cudaMemsetAsync(gs.count, 0, 2 * sizeof(int), s));
     k_cycle_init<<<sb, 64, 0, s>>>(gs, nn, ld, restart, nrhs);
     k_scale_copy<C, C><<<nblocks(vstride), 256, 0, s>>>(V, V, gs.scale, N, nrhs);
@@ -342,18 +461,19 @@ spm_status gmres_cycle(const KrylovOps &ops, int prec, const typename cplx_of<R>
     for (; j < restart && count_host[0] > 0; ++j) {
         C *vj = V + (long)j * vstride;
         w = V + (long)(j + 1) * vstride;
+        SPM_CUDA_TRY(cudaMemsetAsync(gs.count, 0, sizeof(int), s));
         SPM_TRY(ops.apply_A(ops.ctx, prec, vj, w, nrhs, s));       // w = A v_j
         SPM_TRY(ops.apply_Q(ops.ctx, prec, w, tmp, nrhs, s));      // tmp = Q A v_j
         SPM_TRY(ops.solve_S(ops.ctx, prec, tmp, w, nrhs, s));      // w = S^{-1} Q A v_j
         // classical Gram-Schmidt twice, FP64 coefficients
-        SPM_TRY(dots<C>(V, vstride, j + 1, w, N, nrhs, partial, h1, ld, s));
+        SPM_TRY(dots<C>(V, vstride, j + 1, w, N, nrhs, rd, h1, ld, s));
         SPM_TRY(axpy_multi<C>(V, vstride, j + 1, h1, ld, w, N, nrhs, -1.0, s));
-        SPM_TRY(dots<C>(V, vstride, j + 1, w, N, nrhs, partial, h2, ld, s));
-        SPM_TRY(axpy_multi<C>(V, vstride, j + 1, h2, ld, w, N, nrhs, -1.0, s));
-        SPM_TRY(dots<C>(w, vstride, 1, w, N, nrhs, partial, nn, ld, s)); // ||w||^2 (w sits at slot j+1)
-        SPM_CUDA_TRY(cudaMemsetAsync(gs.count, 0, sizeof(int), s));
-        k_arnoldi_givens<<<sb, 64, 0, s>>>(gs, h1, h2, nn, ld, j, restart, nrhs);
-        k_scale_copy<C, C><<<nblocks(vstride), 256, 0, s>>>(w, w, gs.scale, N, nrhs);
+        SPM_TRY(dots<C>(V, vstride, j + 1, w, N, nrhs, rd, h2, ld, s));
+        const int done_groups = j / VGROUP * VGROUP; // all groups but the last
+        SPM_TRY(axpy_multi<C>(V, vstride, done_groups, h2, ld, w, N, nrhs, -1.0, s));
+        launch_pdl(k_arnoldi_end<C>, dim3(dot_blocks(N, nrhs), nrhs), dim3(DOT_THREADS), 0, s, (const C *)V, vstride, done_groups,
+                   j + 1 - done_groups, (const double2 *)h1, (const double2 *)h2, ld, w, N, rd.partial, rd.done, gs, j, restart);
+        launch_pdl(k_scale_copy<C, C>, dim3(nblocks(vstride)), dim3(256), 0, s, w, (const C *)w, (const double *)gs.scale, N, nrhs);
         SPM_CUDA_TRY(cudaMemcpyAsync(count_host, gs.count, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
         SPM_CUDA_TRY(cudaStreamSynchronize(s)); // the only host round trip of an iteration: a convergence count
         ++*iters;
@@ -368,11 +488,9 @@ spm_status gmres_cycle(const KrylovOps &ops, int prec, const typename cplx_of<R>
     return SPM_OK;
 }
 
-template <typename C>
-spm_status norms(const C *v, long N, int nrhs, double2 *partial, double2 *hdev, int ld, std::vector<double> &out,
-                 cudaStream_t s)
+// out[b] = sqrt of the sums of squares that a reduction left in hdev
+spm_status read_norms(const double2 *hdev, int nrhs, int ld, std::vector<double> &out, cudaStream_t s)
 {
-    SPM_TRY(dots<C>(v, 0, 1, v, N, nrhs, partial, hdev, ld, s));
     std::vector<double2> t((size_t)nrhs * ld);
     SPM_CUDA_TRY(cudaMemcpyAsync(t.data(), hdev, sizeof(double2) * nrhs * ld, cudaMemcpyDeviceToHost, s));
     SPM_CUDA_TRY(cudaStreamSynchronize(s));
@@ -393,7 +511,7 @@ spm_status solve_typed(const KrylovOps &ops, const double2 *g, double2 *x, int n
     const int ld = restart + 2;
     // workspace: r (c128), Ax (c128), V (restart+1), d, tmp (inner precision), reductions
     const size_t small = sizeof(double2) * (size_t)nrhs * (3 * ld + (restart + 1) * restart + 2 * restart + restart + 1) +
-                         sizeof(double) * 3 * (size_t)nrhs + sizeof(int) * ((size_t)nrhs + 2);
+                         sizeof(double) * 3 * (size_t)nrhs + sizeof(int) * (2 * (size_t)nrhs + 2);
     size_t bytes = sizeof(double2) * 2 * vstride + sizeof(C) * (size_t)(restart + 3) * vstride +
                    sizeof(double2) * (size_t)nrhs * DOT_BLOCKS * VGROUP + small + 16 * 256;
     DevBuf &ws = *ops.ws; // kept across solves: sized by the largest solve so far
@@ -404,7 +522,8 @@ spm_status solve_typed(const KrylovOps &ops, const double2 *g, double2 *x, int n
     C *V = reinterpret_cast<C *>(p); p += sizeof(C) * (restart + 1) * vstride;
     C *d = reinterpret_cast<C *>(p); p += sizeof(C) * vstride;
     C *tmp = reinterpret_cast<C *>(p); p += sizeof(C) * vstride;
-    double2 *partial = reinterpret_cast<double2 *>(p); p += sizeof(double2) * nrhs * DOT_BLOCKS * VGROUP;
+    Reduce rd;
+    rd.partial = reinterpret_cast<double2 *>(p); p += sizeof(double2) * nrhs * DOT_BLOCKS * VGROUP;
     double2 *hdev = reinterpret_cast<double2 *>(p); p += sizeof(double2) * nrhs * ld;
     double2 *h2dev = reinterpret_cast<double2 *>(p); p += sizeof(double2) * nrhs * ld;
     double2 *nndev = reinterpret_cast<double2 *>(p); p += sizeof(double2) * nrhs * ld;
@@ -418,20 +537,24 @@ spm_status solve_typed(const KrylovOps &ops, const double2 *g, double2 *x, int n
     double *sdev = reinterpret_cast<double *>(p); p += sizeof(double) * nrhs;
     gs.scale = sdev;
     gs.active = reinterpret_cast<int *>(p); p += sizeof(int) * nrhs;
-    gs.count = reinterpret_cast<int *>(p);
+    gs.count = reinterpret_cast<int *>(p); p += sizeof(int) * 2;
+    rd.done = reinterpret_cast<unsigned *>(p);
+    SPM_CUDA_TRY(cudaMemsetAsync(rd.done, 0, sizeof(unsigned) * nrhs, s));
     int count_host[2] = {0, 0};
 
     std::vector<double> gnorm, rnorm, rtol(nrhs), scl(nrhs);
-    SPM_TRY(norms<double2>(g, N, nrhs, partial, hdev, ld, gnorm, s));
+    SPM_TRY(dots<double2>(g, 0, 1, g, N, nrhs, rd, hdev, ld, s));
+    SPM_TRY(read_norms(hdev, nrhs, ld, gnorm, s));
     for (int b = 0; b < nrhs; ++b) if (gnorm[b] == 0.0) gnorm[b] = 1.0;
     int iters = 0, outer = 0;
     double worst = 0.0;
     const double floor_rel = sizeof(R) == 8 ? 1e-14 : 2e-6;
     while (true) {
         SPM_TRY(ops.apply_A(ops.ctx, SPM_C128, x, Ax, nrhs, s));
-        SPM_CUDA_TRY(cudaMemcpyAsync(r, g, sizeof(double2) * vstride, cudaMemcpyDeviceToDevice, s));
-        SPM_TRY(spm_axpby_impl(SPM_C128, vstride, -1.0, Ax, 1.0, r, s)); // r = g - A x
-        SPM_TRY(norms<double2>(r, N, nrhs, partial, hdev, ld, rnorm, s));
+        launch_pdl(k_residual, dim3(dot_blocks(N, nrhs), nrhs), dim3(DOT_THREADS), 0, s, r, g, (const double2 *)Ax, N, rd.partial,
+                   rd.done, hdev, ld);
+        SPM_CUDA_TRY(cudaGetLastError());
+        SPM_TRY(read_norms(hdev, nrhs, ld, rnorm, s));
         worst = 0.0;
         bool done = true;
         for (int b = 0; b < nrhs; ++b) {
@@ -449,13 +572,12 @@ spm_status solve_typed(const KrylovOps &ops, const double2 *g, double2 *x, int n
         if (iters >= maxit) { spm_set_error("no convergence within %d iterations (residual %.3e)", maxit, worst); return SPM_ERR_NO_CONVERGENCE; }
         // inner right-hand side: r / ||r|| in the inner precision
         SPM_CUDA_TRY(cudaMemcpyAsync(sdev, scl.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, s));
-        k_scale_copy<double2, C><<<nblocks(vstride), 256, 0, s>>>(tmp, r, sdev, N, nrhs);
         C *rin = d; // d is free until the cycle writes its result
-        SPM_CUDA_TRY(cudaMemcpyAsync(rin, tmp, sizeof(C) * vstride, cudaMemcpyDeviceToDevice, s));
+        k_scale_copy<double2, C><<<nblocks(vstride), 256, 0, s>>>(rin, r, sdev, N, nrhs);
         int it_cycle = 0;
         int cyc_restart = restart < maxit - iters ? restart : maxit - iters;
         SPM_CUDA_TRY(cudaMemcpyAsync(gs.rtol, rtol.data(), sizeof(double) * nrhs, cudaMemcpyHostToDevice, s));
-        SPM_TRY(gmres_cycle<R>(ops, inner_prec, rin, d, nrhs, cyc_restart, V, tmp, partial, hdev, h2dev, nndev, gs,
+        SPM_TRY(gmres_cycle<R>(ops, inner_prec, rin, d, nrhs, cyc_restart, V, tmp, rd, hdev, h2dev, nndev, gs,
                                count_host, &it_cycle, s));
         iters += it_cycle;
         ++outer;
