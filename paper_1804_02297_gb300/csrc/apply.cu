@@ -85,24 +85,9 @@ constexpr int ZPLAN_FUSED_XY = 8; // plan bit: x and y passes fused per z-plane 
 
 template <int L> __device__ __forceinline__ int xpad(int pos) { return pos + (pos >> 3); }
 
-// asynchronous global -> shared copies (cp.async), BYTES = 8 or 16
-template <int BYTES> __device__ __forceinline__ void cp_async(void *smem, const void *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
-}
-// the same with zero fill: when !valid no byte is read and the BYTES of smem are zeroed
-template <int BYTES> __device__ __forceinline__ void cp_async_zfill(void *smem, const void *gmem, bool valid)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gmem), "n"(BYTES), "r"(valid ? BYTES : 0)
-                 : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// xfwd: w_f of one grid row per line, FFT along x (pruned), 4 fields in turn.
-template <typename R, int L>
+// xfwd: w_f of one grid row per line, FFT along x (pruned), 4 fields in turn, or (APART)
+// one field per block, blockIdx.y.
+template <typename R, int L, bool APART>
 __global__ void __launch_bounds__(256) k2_xfwd(const typename cplx_of<R>::type *__restrict__ x,
                                                const typename cplx_of<R>::type *__restrict__ m,
                                                const typename cplx_of<R>::type *__restrict__ p,
@@ -144,6 +129,7 @@ __global__ void __launch_bounds__(256) k2_xfwd(const typename cplx_of<R>::type *
     }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
+        if (APART && f != (int)blockIdx.y) continue;
         C v[E];
 #pragma unroll
         for (int q = 0; q < H; ++q) {
@@ -546,6 +532,72 @@ __global__ void __launch_bounds__(tx_of<R, L>::v * L / 8) k2_zprod4(typename cpl
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int q = 0; q < 4; ++q) base[d * fs + (long)(t + T * q) * L2] = v[d][q];
+}
+
+// The same on small grids (L <= 32), a line per thread group: a quarter of the block's
+// threads per field, TX adjacent columns.  The groups transform their fields side by side,
+// a warp each; p.E's transform goes to the other three through shared
+// memory; they form the product and transform back.  Four times the warps, each with two
+// transforms instead of seven one after another: in complex128 a warp's FP64 instruction
+// takes 64 cycles, and at n = 16 the four-line kernel is 128 warps on 608 schedulers
+// (33.9 us; this one 14.3; n = 8 28.7 and 12.3; complex64 6.8 and 5.8).  From L = 64 on the
+// four-line kernel has warps enough and shares its twiddles and spectra between the
+// fields (complex64 n = 64: 30.7 against 45.1 us, complex128 567 against 590).
+template <typename R, int L> struct zfl {
+    using C = typename cplx_of<R>::type;
+    static constexpr int T = L / 8;
+    static constexpr int TX = 32 / T; // a warp per field
+    static_assert(L <= 32, "small grids");
+    static constexpr int GROUP = TX * T, THREADS = 4 * GROUP;
+    static constexpr size_t smem = sizeof(C) * 4 * L * TX;
+};
+template <typename R, int L>
+__global__ void __launch_bounds__(zfl<R, L>::THREADS) k2_zfield(typename cplx_of<R>::type *W2,
+                                                                  const typename cplx_of<R>::type *__restrict__ spec,
+                                                             const typename cplx_of<R>::type *__restrict__ tw)
+{
+    pdl_wait_and_trigger();
+    using C = typename cplx_of<R>::type;
+    constexpr int T = zfl<R, L>::T, TX = zfl<R, L>::TX, GROUP = zfl<R, L>::GROUP, n = L / 2, n1 = n + 1;
+    constexpr long L2 = (long)L * L, oct = (long)n1 * n1 * n1, fs = (long)n * L * L;
+    extern __shared__ unsigned char smem_raw[];
+    C *sm = reinterpret_cast<C *>(smem_raw); // 4 exchange buffers [4][L][TX]
+    const int f = threadIdx.x / GROUP, tid = threadIdx.x % GROUP, c = tid % TX, t = tid / TX;
+    const long col = (long)blockIdx.x * TX + c;
+    C *base = W2 + (long)blockIdx.y * 4 * fs + f * fs + col;
+    C *own = sm + f * L * TX;
+    auto buf = [&](int pos) -> C & { return own[pos * TX + c]; };
+    auto sync = [&]() { __syncwarp(); }; // a group is a warp
+    static_assert(GROUP == 32, "one warp per field");
+    C v[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = base[(long)(t + T * q) * L2];
+#pragma unroll
+    for (int q = 4; q < 8; ++q) v[q] = czero<C>();
+    fftr::fft_line<-1, L, true>(v, t, buf, sync, tw);
+    C *w4 = sm + 3 * L * TX; // group 3's buffer; its last exchange has been read
+    if (f == 3) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w4[(t + T * q) * TX + c] = v[q];
+    }
+    __syncthreads();
+    if (f == 3) return;
+    const int eta = (int)(col / L), xi = (int)(col % L);
+    const int a1 = xi <= n ? xi : L - xi, a2 = eta <= n ? eta : L - eta;
+    const C *Kf = spec + (long)a2 * n1 + a1;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int zeta = t + T * q;
+        const int o = (zeta <= n ? zeta : L - zeta) * n1 * n1;
+        const C K0 = Kf[o];
+        C Kd = Kf[(1 + f) * oct + o];
+        const int fr = f == 0 ? xi : (f == 1 ? eta : zeta);
+        if (fr > n) { Kd.x = -Kd.x; Kd.y = -Kd.y; }
+        v[q] = cfma(K0, v[q], cmul(Kd, w4[zeta * TX + c]));
+    }
+    fftr::fft_line<1, L, false>(v, t, buf, sync, tw);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) base[(long)(t + T * q) * L2] = v[q];
 }
 
 // Exchange buffer of a 16-per-thread line shared by TX columns: position pos of
@@ -1061,10 +1113,11 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     // rows per block: 256 threads, fewer (down to a warp) while that leaves under two
     // blocks for each of 152 SMs: x-forward at n = 16 in complex128 was 4 blocks and
     // 40 us, with 32 it takes 21
-    auto launch_rows = [&](auto kernel, long rows, auto... args) {
+    auto launch_rows = [&](auto kernel, long rows, int fields, auto... args) {
         int lines = LPB;
         while (lines % 2 == 0 && lines * T >= 64 && (rows + lines - 1) / lines < 2 * 152) lines /= 2;
-        launch_pdl(kernel, dim3((unsigned)((rows + lines - 1) / lines)), dim3(lines * T), sizeof(C) * lines * (L + L / 8), s, args...);
+        launch_pdl(kernel, dim3((unsigned)((rows + lines - 1) / lines), fields), dim3(lines * T), sizeof(C) * lines * (L + L / 8), s,
+                   args...);
     };
     const bool fused = (zvar & ZPLAN_FUSED_XY) != 0; // x and y passes fused per z-plane
     zvar &= ZPLAN_FUSED_XY - 1;
@@ -1072,7 +1125,8 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     constexpr size_t sm_zprod4 = 4 * sm_cols;
     static bool attrs = false;
     if (!attrs) {
-        allow_smem(k2_xfwd<R, L>, sm_rows);
+        allow_smem(k2_xfwd<R, L, true>, sm_rows);
+        allow_smem(k2_xfwd<R, L, false>, sm_rows);
         allow_smem(k2_xinv<R, L>, sm_rows);
         allow_smem(k2_cols<R, L, -1, true>, sm_cols);
         allow_smem(k2_cols<R, L, 1, false>, sm_cols);
@@ -1102,7 +1156,10 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     }
     if (!fused_done) {
         long rows = (long)nb * n2;
-        launch_rows(k2_xfwd<R, L>, rows, xb, m, p, W1, (int)rows, tw);
+        // too few rows for a warp on every scheduler (4 x 152): the fields apart (n = 16 in
+        // complex128: 20 us one after another)
+        if (rows * T < 32 * 4 * 152) launch_rows(k2_xfwd<R, L, true>, rows, 4, xb, m, p, W1, (int)rows, tw);
+        else launch_rows(k2_xfwd<R, L, false>, rows, 1, xb, m, p, W1, (int)rows, tw);
         mark();
         if constexpr (line_elems(L) == 8 && n % 2 == 0)
             launch_pdl(k2_cols2<R, L, -1, true>, dim3(L / TX, n / 2, nb * 4), dim3(THR), 2 * sm_cols, s, (const C *)W1,
@@ -1158,7 +1215,11 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     }
     if constexpr (line_elems(L) == 8) {
         if (!done && zvar == ZPROD_FOUR) {
-            launch_pdl(k2_zprod4<R, L>, dim3((unsigned)(L2 / TX), nb), dim3(THR), sm_zprod4, s, W2, spec, tw);
+            if constexpr (L <= 32)
+                launch_pdl(k2_zfield<R, L>, dim3((unsigned)(L2 / zfl<R, L>::TX), nb), dim3(zfl<R, L>::THREADS), zfl<R, L>::smem,
+                           s, W2, spec, tw);
+            else
+                launch_pdl(k2_zprod4<R, L>, dim3((unsigned)(L2 / TX), nb), dim3(THR), sm_zprod4, s, W2, spec, tw);
             done = true;
         }
     }
@@ -1179,7 +1240,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     mark();
     {
         long rows = (long)nb * 3 * n2;
-        launch_rows(k2_xinv<R, L>, rows, (const C *)W1, xb, yb, rows, tw);
+        launch_rows(k2_xinv<R, L>, rows, 1, (const C *)W1, xb, yb, rows, tw);
     }
     mark();
     return SPM_OK;
@@ -1593,29 +1654,33 @@ __global__ void __launch_bounds__(Q_THREADS) k_q(const float2 *__restrict__ v,
 // nearly free beside that, and what counts is that every SM gets the same share of full
 // warps: the 32 x 4 x 4 tiles of the complex64 kernel left one tile's work on each of 16
 // SMs at n = 16 (157 us; this kernel 17 us) and half-empty tiles elsewhere (n = 64: 600
-// against 421 us, n = 96: 1780 against 1395 us).  In complex64 the tiles win from n = 16
+// against 416 us, n = 96: 1780 against 1395 us).  In complex64 the tiles win from n = 16
 // on (n = 64: 21 against 33 us) and the two are equal below.
-template <typename C>
-__global__ void __launch_bounds__(Q_THREADS) k_q_direct(const C *__restrict__ v, const C *__restrict__ qtab,
-                                                        C *__restrict__ y, int n)
+// SPLIT = 3, for grids of fewer warps than schedulers: the three components d of a point
+// in three warps of a block, their sums joined through shared memory.
+template <typename C, int SPLIT>
+__global__ void __launch_bounds__(SPLIT == 1 ? Q_THREADS : 96) k_q_direct(const C *__restrict__ v, const C *__restrict__ qtab,
+                                                                         C *__restrict__ y, int n)
 {
     pdl_wait_and_trigger();
+    constexpr int PTS = SPLIT == 1 ? Q_THREADS : 32; // points per block
     const int n2 = n * n, n3 = n2 * n;
-    const int i = blockIdx.x * Q_THREADS + threadIdx.x, c = blockIdx.y;
-    if (i >= n3) return;
+    const int i = blockIdx.x * PTS + threadIdx.x % PTS, c = blockIdx.y, d0 = threadIdx.x / PTS;
+    const bool ok = i < n3;
+    if (SPLIT == 1 && !ok) return;
     const int i1 = i % n, i2 = (i / n) % n, i3 = i / n2;
     const bool lo[3] = {i1 > 0, i2 > 0, i3 > 0}, hi[3] = {i1 < n - 1, i2 < n - 1, i3 < n - 1};
     const int cls = (lo[0] ? (hi[0] ? 1 : 2) : 0) + 3 * (lo[1] ? (hi[1] ? 1 : 2) : 0) + 9 * (lo[2] ? (hi[2] ? 1 : 2) : 0);
-    const C *al = qtab + cls * 243 + c;
-    const C *vb = v + (long)blockIdx.z * 3 * n3 + i;
+    const C *al = qtab + cls * 243 + c + d0 * 81;
+    const C *vb = v + ((long)blockIdx.z * 3 + d0) * n3 + i;
     C acc = czero<C>();
 #pragma unroll 1
-    for (int d = 0; d < 3; ++d, vb += n3, al += 81) {
+    for (int d = 0; d < 3 / SPLIT; ++d, vb += n3, al += 81) {
         C a[27], u[27]; // all loads of a component before its FMAs
 #pragma unroll
         for (int o = 0; o < 27; ++o) {
             const int o1 = o % 3 - 1, o2 = (o / 3) % 3 - 1, o3 = o / 9 - 1;
-            const bool in = (o1 == 0 || (o1 < 0 ? lo[0] : hi[0])) && (o2 == 0 || (o2 < 0 ? lo[1] : hi[1])) &&
+            const bool in = ok && (o1 == 0 || (o1 < 0 ? lo[0] : hi[0])) && (o2 == 0 || (o2 < 0 ? lo[1] : hi[1])) &&
                             (o3 == 0 || (o3 < 0 ? lo[2] : hi[2]));
             a[o] = al[3 * o];
             u[o] = czero<C>();
@@ -1623,6 +1688,13 @@ __global__ void __launch_bounds__(Q_THREADS) k_q_direct(const C *__restrict__ v,
         }
 #pragma unroll
         for (int o = 0; o < 27; ++o) acc = cfma(a[o], u[o], acc);
+    }
+    if constexpr (SPLIT == 3) {
+        __shared__ C part[2][32];
+        if (d0 > 0) part[d0 - 1][threadIdx.x % 32] = acc;
+        __syncthreads();
+        if (d0 > 0 || !ok) return;
+        acc = acc + part[0][threadIdx.x] + part[1][threadIdx.x];
     }
     y[((long)blockIdx.z * 3 + c) * n3 + i] = acc;
 }
@@ -1634,10 +1706,16 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
     const int n = P->n;
     const C *qtab = sizeof(R) == 8 ? P->qtab128.as<C>() : P->qtab64.as<C>();
     if constexpr (sizeof(R) == 8) {
-        const dim3 grid((unsigned)((n * n * n + Q_THREADS - 1) / Q_THREADS), 3, (unsigned)nrhs);
-        static const EvenPlacement even(k_q_direct<C>, Q_THREADS);
-        launch_pdl(k_q_direct<C>, grid, dim3(Q_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, (const C *)vv,
-                   qtab, (C *)yv, n);
+        // by n alone, so that a block of right-hand sides gives the bits of single ones
+        if (3 * n * n * n <= 32 * 4 * 152) {
+            launch_pdl(k_q_direct<C, 3>, dim3((unsigned)((n * n * n + 31) / 32), 3, (unsigned)nrhs), dim3(96), 0, s, (const C *)vv,
+                       qtab, (C *)yv, n);
+        } else {
+            const dim3 grid((unsigned)((n * n * n + Q_THREADS - 1) / Q_THREADS), 3, (unsigned)nrhs);
+            static const EvenPlacement even(k_q_direct<C, 1>, Q_THREADS);
+            launch_pdl(k_q_direct<C, 1>, grid, dim3(Q_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, (const C *)vv,
+                       qtab, (C *)yv, n);
+        }
         SPM_CUDA_TRY(cudaGetLastError());
         return SPM_OK;
     } else {

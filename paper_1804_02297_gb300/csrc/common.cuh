@@ -99,6 +99,23 @@ static inline int ilog2(int v)
     return r;
 }
 
+// ------------------------------------------------------------ asynchronous copies
+// asynchronous global -> shared copies (cp.async), BYTES = 4, 8 or 16
+template <int BYTES> __device__ __forceinline__ void cp_async(void *smem, const void *gmem)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(sa), "l"(gmem), "n"(BYTES) : "memory");
+}
+// the same with zero fill: when !valid no byte is read and the BYTES of smem are zeroed
+template <int BYTES> __device__ __forceinline__ void cp_async_zfill(void *smem, const void *gmem, bool valid)
+{
+    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gmem), "n"(BYTES), "r"(valid ? BYTES : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
 // ------------------------------------------------------------ dependent launches
 // Programmatic dependent launch (sm_90 and later).  The passes of an apply are
 // launched with programmatic stream serialization: each pass kernel triggers its
