@@ -533,14 +533,16 @@ inline unsigned blocks(long cnt, int t = 256) { return (unsigned)((cnt + t - 1) 
 //   forward, deepest level first:  [y; t] = G w_own,  Y_own = y,  W_bnd -= t
 //   backward, root first:          Y_own -= X Y_bnd
 // One launch per level and direction.  Every node's matrix (column-major, ld rows)
-// is cut into tiles of at most ST_ROWS x ST_COLS entries; a block of 256 threads
-// owns one tile: thread t takes row t % nrow and the columns t / nrow + groups k,
+// is cut into tiles of at most st_elems entries, copied to shared memory; a block of 256
+// threads owns one tile: thread t takes row t % nrow and the columns t / nrow + groups k,
 // groups = 256 / nrow, so that a tile of 49 rows keeps 245 threads busy.
 // Bound: complex64 by reading the factor; complex128 by the FP64 pipe (4 FMAs per
 // 16 bytes at 1.25 TFLOP/s: 2.5 TB/s); small grids by the 2 x levels dependent
-// launches.  Against the packing, GEMV and scatter launches this replaced (four per
-// level and direction), S^-1 Q took: 2-D n = 239 complex128 528 us (2017 before),
-// 3-D n = 32 complex64 385 us (1075 before), 16 right-hand sides 1244 us (2932).
+// launches (3.3 us each at n = 16).  S^-1, against the packing, GEMV and scatter launches
+// this replaced (four per level and direction): 2-D complex128 n = 119 139 us (1063
+// before), n = 239 294 (1970; 137 by the FP64 pipe); 3-D complex64 n = 16 40 (378), n = 32
+// 314 (1067; 219 by the factor's bytes), n = 64 4090 (4655); 16 right-hand sides n = 16 222
+// (1439), n = 32 1072 (2887; 300 by the FP32 pipe), n = 64 13200 (22170).
 struct SolveTile {
     long mat, scale;  // first entry of the tile; scale of its first column (half storage)
     int ld, nrow, ncol;
@@ -549,12 +551,18 @@ struct SolveTile {
     int bout;         // place of row nown in the boundary list
     int full;         // the tile spans every column: no other block adds to its own rows
 };
-constexpr int ST_THREADS = 256, ST_COLS = 256, ST_GROUPS = 16;
+constexpr int ST_THREADS = 256, ST_GROUPS = 16;
+// Tiles go through shared memory whole (cp.async) in complex128, where the registers are
+// better spent on more warps for the FP64 pipe (n = 239: 339 us against 500), and in
+// complex64 for factors that stay in the L2 (3-D n = 16: 43 us against 63); larger ones
+// stream through registers, eight entries ahead (n = 64: 4.49 ms against 5.43).
+constexpr size_t ST_STAGED_BYTES = 256u << 20;
 template <typename C> constexpr int st_rows() { return 1024 / (int)sizeof(C); } // 1 KB of each column
+template <typename C> constexpr int st_elems() { return sizeof(C) == 8 ? 6144 : 2048; } // of a staged tile: 48, 32 KB
 
-__device__ __forceinline__ float2 load_as(const float2 *p) { return __ldcs(p); }
-__device__ __forceinline__ double2 load_as(const double2 *p) { return __ldcs(p); }
-__device__ __forceinline__ float2 load_as(const __half2 *p) { return __half22float2(__ldcs(p)); }
+__device__ __forceinline__ float2 value_of(float2 v) { return v; }
+__device__ __forceinline__ double2 value_of(double2 v) { return v; }
+__device__ __forceinline__ float2 value_of(__half2 v) { return __half22float2(v); }
 
 __device__ __forceinline__ void add_to(float2 *p, float2 v) { atomicAdd(p, v); }
 __device__ __forceinline__ void add_to(double2 *p, double2 v)
@@ -598,37 +606,58 @@ template <int NB> struct TileAcc<float2, NB> {
     __device__ __forceinline__ float2 get(int b) const { return make_float2(p[b].x - q[b].y, p[b].y + q[b].x); }
 };
 
-template <typename C, typename S, int NB, bool FWD>
-__global__ void __launch_bounds__(ST_THREADS) k_nd_level(const S *__restrict__ M, const float *__restrict__ scales,
+// Blocks per SM that the registers are held to.  complex64, one right-hand side: loads in
+// flight against blocks to overlap their starts and ends (3-D n = 32: four 392 us, five
+// 346, six 314, eight, which spill, 562; n = 64: 4.60, 3.94, 4.09, 6.46 ms).  Several wait on
+// shared memory between their packed FMAs and gain from warps (8 of them at n = 32: one
+// block 1050 us, two 686, three 606, four 586; 16, whose sums alone are 64 registers: one
+// 1599, two 1072, three 1585).  complex128 (2-D n = 239): one right-hand side four 342 us,
+// five 312, six 294, eight 343; four 843, 840, 870, 884; eight 1802 with two, 1680 with four.
+template <typename C, int NB> constexpr int st_blocks()
+{
+    if (sizeof(C) == 16) return NB <= 2 ? 6 : (NB == 4 ? 5 : 4);
+    return NB <= 2 ? 6 : (NB <= 8 ? 4 : 2);
+}
+
+template <typename C, typename S, int NB, bool FWD, bool STAGED>
+__global__ void __launch_bounds__(ST_THREADS, st_blocks<C, NB>()) k_nd_level(const S *__restrict__ M, const float *__restrict__ scales,
                                                          const SolveTile *__restrict__ tiles,
-                                                         const int *__restrict__ bnd, C *W, C *Y, int nrhs)
+                                                         const int *__restrict__ bnd, C *W, C *Y, int nrhs, int tile_elems)
 {
     constexpr bool SCALED = !std::is_same<S, C>::value;
-    constexpr int UNR = NB >= 16 ? 4 : 8; // matrix entries a thread has in flight
-    __shared__ __align__(16) C xs[(ST_COLS > ST_THREADS ? ST_COLS : ST_THREADS) * NB];
+    constexpr int UNR = STAGED ? 1 : (NB == 8 ? 4 : 8); // matrix entries a thread has in flight in registers
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    S *ts = reinterpret_cast<S *>(smem_raw); // the tile, [ncol][nrow]
+    C *xs = reinterpret_cast<C *>(smem_raw + (STAGED ? sizeof(S) * (size_t)tile_elems : 0)); // columns, then sums
     const SolveTile tl = tiles[blockIdx.x];
     const int groups = min(ST_THREADS / tl.nrow, ST_GROUPS);
     const int row = threadIdx.x % tl.nrow, g = threadIdx.x / tl.nrow;
     const bool act = g < groups;
-    const S *mrow = M + tl.mat + row;
+    const S *src = M + tl.mat + row;
     const int steps = (tl.ncol + groups - 1) / groups; // columns per thread
-    C cur[UNR];
+    S cur[UNR];
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int k = 0; k < UNR; ++k) {
             const int c = g + (k0 + k) * groups;
-            cur[k] = act && c < tl.ncol ? load_as(mrow + (long)c * tl.ld) : czero<C>();
+            if (act && c < tl.ncol) cur[k] = __ldcs(src + (long)c * tl.ld);
         }
     };
-    // the factor does not change: the first entries are fetched before the previous
-    // level's results are waited for
-    fetch(0);
+    // the factor does not change: the tile is on its way before the previous level's
+    // results are waited for.  A thread copies the entries that it multiplies.
+    if constexpr (STAGED) {
+        if (act)
+            for (int c = g; c < tl.ncol; c += groups) cp_async<sizeof(S)>(&ts[c * tl.nrow + row], src + (long)c * tl.ld);
+        cp_async_commit();
+    } else {
+        fetch(0);
+    }
     pdl_wait_and_trigger();
     for (int b0 = 0; b0 < nrhs; b0 += NB) {
         const int nb = min(NB, nrhs - b0);
         if (b0 > 0) {
             __syncthreads(); // the sums of the previous group have been read
-            fetch(0);
+            if constexpr (!STAGED) fetch(0);
         }
         for (int i = threadIdx.x; i < tl.ncol * NB; i += ST_THREADS) {
             const int c = i / NB, b = i % NB;
@@ -639,18 +668,26 @@ __global__ void __launch_bounds__(ST_THREADS) k_nd_level(const S *__restrict__ M
             }
             xs[i] = v;
         }
+        if constexpr (STAGED) cp_async_wait<0>();
         __syncthreads();
         TileAcc<C, NB> acc;
         acc.clear();
-        for (int k0 = 0; k0 < steps; k0 += UNR) {
-            C now[UNR];
+        if constexpr (STAGED) {
+            if (act) {
+#pragma unroll 4
+                for (int c = g; c < tl.ncol; c += groups) acc.mac(value_of(ts[c * tl.nrow + row]), xs + c * NB);
+            }
+        } else {
+            for (int k0 = 0; k0 < steps; k0 += UNR) {
+                S now[UNR];
 #pragma unroll
-            for (int k = 0; k < UNR; ++k) now[k] = cur[k];
-            if (k0 + UNR < steps) fetch(k0 + UNR);
+                for (int k = 0; k < UNR; ++k) now[k] = cur[k];
+                if (k0 + UNR < steps) fetch(k0 + UNR);
 #pragma unroll
-            for (int k = 0; k < UNR; ++k) {
-                const int c = g + (k0 + k) * groups;
-                if (c < tl.ncol) acc.mac(now[k], xs + c * NB);
+                for (int k = 0; k < UNR; ++k) {
+                    const int c = g + (k0 + k) * groups;
+                    if (act && c < tl.ncol) acc.mac(value_of(now[k]), xs + c * NB);
+                }
             }
         }
         __syncthreads();
@@ -762,6 +799,8 @@ struct NDFactor {
         int ntiles_f, ntiles_b;
     };
     std::vector<Level> levels;
+    int tile_elems = 0, tile_cols = 0; // of the largest tiles
+    bool staged = false;               // tiles copied to shared memory whole
     DevBuf st_tiles, st_bnd, st_rank, st_point; // tiles, boundary unknowns, rank of each point and back
     DenseWork *dense = nullptr; // Gauss-Jordan workspace
     ~NDFactor()
@@ -830,13 +869,15 @@ int build_tree(std::vector<Node> &nodes, const int lo[3], const int hi[3], int v
 
 // Elimination ranks, boundary lists and tiles of every level.  A level's tiles hold
 // at most st_rows rows (a node's rows are cut evenly) and as many columns as leave
-// about eight tiles for every SM, between 8 and ST_COLS: levels of few nodes spread
-// over the chip, levels of many read long stretches and add each row's sum once.
+// about five tiles for every SM (four or eight are 1 to 4 % slower), 8 to 256 of them and
+// at most st_elems entries if staged: levels of few nodes spread over the chip, levels of
+// many add each row's sum less often.
 template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std::vector<int> &pts)
 {
     using C = typename cplx_of<R>::type;
     const std::vector<Node> &nodes = F->nodes;
     const int NN = (int)nodes.size(), D = F->D;
+    F->staged = sizeof(R) == 8 || F->stored_bytes <= ST_STAGED_BYTES;
     std::vector<int> rank(F->npts), point(F->npts), bnd;
     std::vector<int> base(NN), boff(NN);
     int next = 0;
@@ -866,14 +907,14 @@ template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std
             const double o = D * (double)nodes[id].nown, b = D * (double)nodes[id].nbnd;
             level += fwd ? (o + b) * o : o * b;
         }
-        const double per_tile = level / (8 * 152);
+        const double per_tile = level / (5 * 152);
         for (int id : ids) {
             const Node &nd = nodes[id];
             const int o = D * nd.nown, b = D * nd.nbnd;
             const int rows = fwd ? o + b : o, cols = fwd ? o : b;
             if (cols == 0) continue;
             const int nr = (rows + st_rows<C>() - 1) / st_rows<C>(), rt = (rows + nr - 1) / nr;
-            int ct = (int)std::min<double>(ST_COLS, std::max(8.0, per_tile / rt));
+            int ct = std::min({ST_THREADS, std::max(1, F->staged ? st_elems<C>() / rt : ST_THREADS), (int)std::min(1e6, std::max(8.0, per_tile / rt))});
             const int nc = (cols + ct - 1) / ct;
             ct = (cols + nc - 1) / nc;
             for (int r0 = 0; r0 < rows; r0 += rt)
@@ -889,6 +930,8 @@ template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std
                     t.nown = std::max(0, std::min(t.nrow, o - r0));
                     t.bout = boff[id] + std::max(0, r0 - o);
                     t.full = t.ncol == cols;
+                    F->tile_elems = std::max(F->tile_elems, t.nrow * t.ncol);
+                    F->tile_cols = std::max(F->tile_cols, t.ncol);
                     tt.push_back(t);
                 }
         }
@@ -1346,35 +1389,60 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
     return build_solve_tiles<R>(F, pts);
 }
 
-template <typename C, typename S, int NB>
+// forward, deepest level first; backward, root first: launch(kernel of the direction, tiles, count)
+template <typename KF, typename KB, typename L>
+static void each_level(NDFactor *F, KF fwd, KB bwd, L launch)
+{
+    const SolveTile *tiles = F->st_tiles.as<const SolveTile>();
+    const int NL = (int)F->levels.size();
+    for (int l = 0; l < NL; ++l)
+        if (F->levels[l].ntiles_f > 0) launch(fwd, tiles + F->levels[l].tiles_f, F->levels[l].ntiles_f);
+    for (int l = NL - 1; l >= 0; --l)
+        if (F->levels[l].ntiles_b > 0) launch(bwd, tiles + F->levels[l].tiles_b, F->levels[l].ntiles_b);
+}
+
+// Opt in to the shared memory (a failure shows as a failed launch), and, where tiles stream
+// through registers, ask for the L1: lines in flight live there, and without a request the
+// SM keeps the division that the kernel before it wanted (S^-1 at n = 32: 314 us among its
+// like, 440 after Q).
+template <typename K> static bool opt_in(K kernel, bool staged, int percent)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) == cudaSuccess &&
+           (staged || cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, percent) == cudaSuccess);
+}
+
+template <typename C, typename S, int NB, bool STAGED>
 static void launch_levels(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStream_t s)
 {
-    const float *scales = F->scales.as<float>();
-    const SolveTile *tiles = F->st_tiles.as<SolveTile>();
-    const int *bnd = F->st_bnd.as<int>(), NL = (int)F->levels.size();
-    for (int l = 0; l < NL; ++l) { // forward, deepest level first
-        const NDFactor::Level &lv = F->levels[l];
-        if (lv.ntiles_f > 0)
-            launch_pdl(k_nd_level<C, S, NB, true>, dim3(lv.ntiles_f), dim3(ST_THREADS), 0, s, M, scales, tiles + lv.tiles_f,
-                       bnd, W, Y, nrhs);
-    }
-    for (int l = NL - 1; l >= 0; --l) { // backward, root first
-        const NDFactor::Level &lv = F->levels[l];
-        if (lv.ntiles_b > 0)
-            launch_pdl(k_nd_level<C, S, NB, false>, dim3(lv.ntiles_b), dim3(ST_THREADS), 0, s, M, scales, tiles + lv.tiles_b,
-                       bnd, W, Y, nrhs);
-    }
+    // percent of 228 KB for the blocks that fit: NB x 256 sums and a reserved kilobyte each
+    constexpr int percent = st_blocks<C, NB>() * ((int)sizeof(C) * NB * ST_THREADS + 1024) / 2334 + 1;
+    static const bool allowed = opt_in(k_nd_level<C, S, NB, true, STAGED>, STAGED, percent) &&
+                                opt_in(k_nd_level<C, S, NB, false, STAGED>, STAGED, percent);
+    (void)allowed;
+    // at most a 48 KB tile and 32 KB of sums
+    const size_t smem = (STAGED ? sizeof(S) * (size_t)F->tile_elems : 0) + sizeof(C) * NB * std::max(ST_THREADS, F->tile_cols);
+    each_level(F, k_nd_level<C, S, NB, true, STAGED>, k_nd_level<C, S, NB, false, STAGED>, [&](auto kernel, const SolveTile *t, int n) {
+        launch_pdl(kernel, dim3(n), dim3(ST_THREADS), smem, s, M, (const float *)F->scales.as<float>(), t,
+                   F->st_bnd.as<const int>(), W, Y, nrhs, F->tile_elems);
+    });
 }
 
 // right-hand sides per pass over a tile: a tile is read once per group of NB
 template <typename C, typename S>
 static void launch_solve(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStream_t s)
 {
-    if (nrhs == 1) launch_levels<C, S, 1>(F, M, W, Y, nrhs, s);
-    else if (nrhs == 2) launch_levels<C, S, 2>(F, M, W, Y, nrhs, s);
-    else if (nrhs <= 4) launch_levels<C, S, 4>(F, M, W, Y, nrhs, s);
-    else if (nrhs <= 8 || sizeof(C) == 16) launch_levels<C, S, 8>(F, M, W, Y, nrhs, s);
-    else launch_levels<C, S, sizeof(C) == 16 ? 8 : 16>(F, M, W, Y, nrhs, s);
+    constexpr bool DBL = sizeof(C) == 16;
+    if (nrhs > 8 && !DBL) launch_levels<C, S, DBL ? 8 : 16, DBL>(F, M, W, Y, nrhs, s);
+    else if (nrhs > 4) launch_levels<C, S, 8, DBL>(F, M, W, Y, nrhs, s);
+    else if (F->staged) {
+        if (nrhs == 1) launch_levels<C, S, 1, true>(F, M, W, Y, nrhs, s);
+        else if (nrhs == 2) launch_levels<C, S, 2, true>(F, M, W, Y, nrhs, s);
+        else launch_levels<C, S, 4, true>(F, M, W, Y, nrhs, s);
+    } else {
+        if (nrhs == 1) launch_levels<C, S, 1, DBL>(F, M, W, Y, nrhs, s);
+        else if (nrhs == 2) launch_levels<C, S, 2, DBL>(F, M, W, Y, nrhs, s);
+        else launch_levels<C, S, 4, DBL>(F, M, W, Y, nrhs, s);
+    }
 }
 
 template <typename R>
