@@ -180,13 +180,17 @@ template <int L> struct Geo2 {
 // memory (coalesced across columns), the three fields transformed along x2
 // together (input rows >= n are the zero padding; the three lines share every
 // barrier), the L frequencies back through shared memory to W[b][f][v2][i1]
-// (rows of length n, coalesced across columns).
-template <typename R, int L>
+// (rows of length n, coalesced across columns).  NF = 1: one field per block, blockIdx.z
+// (complex128, bound by the FP64 pipe: 3 n units of work share out over the SMs where n
+// columns leave the last of three or four rounds nearly empty: n = 479 105 -> 87 us here,
+// 81 -> 59 in pass 3).
+template <typename R, int L, int NF>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
     k2d_colfwd(const typename cplx_of<R>::type *__restrict__ x, const typename cplx_of<R>::type *__restrict__ m,
                const typename cplx_of<R>::type *__restrict__ p, typename cplx_of<R>::type *__restrict__ W, int n,
                const typename cplx_of<R>::type *__restrict__ tw, int COLS)
 {
+    pdl_wait_and_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int T = L / 8, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
@@ -196,6 +200,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
     const long b = blockIdx.y, N = (long)n * n;
     const C *xb = x + b * 2 * N;
     const long fsm = (long)COLS * LS;
+    const int f0 = NF == 1 ? blockIdx.z : 0; // the first of the block's fields
     auto buf = [&](int k, int pos) -> C & { return sm[k * fsm + c * LS + pad8(pos)]; };
     auto sync = [&]() { __syncthreads(); };
     // every thread stages at most 4 points (COLS * n <= COLS * L / 2 = 4 blockDim.x):
@@ -222,16 +227,19 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
             const int cc = i & (COLS - 1), r = i / COLS;
             if (r < n) {
                 const int at = cc * LS + pad8(r);
-                sm[at] = cmul(mm[q], e0[q]);
-                sm[fsm + at] = cmul(mm[q], e1[q]);
-                sm[2 * fsm + at] = cfma(p0[q], e0[q], cmul(p1[q], e1[q]));
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    if (NF == 1 && k != f0) continue;
+                    sm[(NF == 1 ? 0 : k) * fsm + at] = k == 0 ? cmul(mm[q], e0[q])
+                                                              : (k == 1 ? cmul(mm[q], e1[q]) : cfma(p0[q], e0[q], cmul(p1[q], e1[q])));
+                }
             }
         }
     }
     __syncthreads();
-    C v[3][8];
+    C v[NF][8];
 #pragma unroll
-    for (int f = 0; f < 3; ++f)
+    for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int r = t + T * q;
@@ -239,14 +247,14 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
             v[f][q + 4] = czero<C>();
         }
     __syncthreads();
-    fftr::fft_lines<-1, L, true, 3>(v, t, buf, sync, tw);
+    fftr::fft_lines<-1, L, true, NF>(v, t, buf, sync, tw);
 #pragma unroll
-    for (int f = 0; f < 3; ++f)
+    for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int q = 0; q < 8; ++q) buf(f, t + T * q) = v[f][q];
     __syncthreads();
-    for (int f = 0; f < 3; ++f) {
-        C *Wf = W + (b * 3 + f) * (long)L * n;
+    for (int f = 0; f < NF; ++f) {
+        C *Wf = W + (b * 3 + f0 + f) * (long)L * n;
 #pragma unroll
         for (int q = 0; q < 8; ++q) { // COLS * L = 8 blockDim.x
             const int i = q * blockDim.x + threadIdx.x;
@@ -266,6 +274,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k2d_rowprod(typen
                                                    const typename cplx_of<R>::type *__restrict__ spec, int n,
                                                    const typename cplx_of<R>::type *__restrict__ tw, int RB)
 {
+    pdl_wait_and_trigger();
     using C = typename cplx_of<R>::type;
     using G = Geo2<L>;
     constexpr int T = G::T, H = L / 2 + 1;
@@ -292,15 +301,15 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k2d_rowprod(typen
         }
     fftr::fft_lines<-1, L, true, 3>(v, t, buf, sync, tw);
     const int a2 = v2 <= L / 2 ? v2 : L - v2;
-    const R s2 = v2 > L / 2 ? (R)-1 : (R)1;
     const C *K0 = spec + (long)a2 * H, *K1 = K0 + (long)H * H, *K2 = K1 + (long)H * H;
     C y[2][8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const int v1 = t + T * q;
         const int a1 = v1 <= L / 2 ? v1 : L - v1;
-        const R s1 = v1 > L / 2 ? (R)-1 : (R)1;
-        const C k0 = K0[a1], k1 = cscale(K1[a1], s1), k2 = cscale(K2[a1], s2);
+        C k0 = K0[a1], k1 = K1[a1], k2 = K2[a1];
+        if (v1 > L / 2) { k1.x = -k1.x; k1.y = -k1.y; } // a sign costs no multiplication
+        if (v2 > L / 2) { k2.x = -k2.x; k2.y = -k2.y; }
         y[0][q] = cfma(k0, v[0][q], cmul(k1, v[2][q]));
         y[1][q] = cfma(k0, v[1][q], cmul(k2, v[2][q]));
     }
@@ -317,13 +326,14 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k2d_rowprod(typen
 // Pass 3, one column i1 < n per line, COLS adjacent columns per block: the
 // L rows of fields 0, 1 staged in shared memory (coalesced across columns),
 // both inverse FFTs along x2 together, rows i2 < n back through shared memory,
-// y = x + result.
-template <typename R, int L>
+// y = x + result.  NF = 1: one field per block, as in pass 1.
+template <typename R, int L, int NF>
 __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
     k2d_colinv(const typename cplx_of<R>::type *__restrict__ W, const typename cplx_of<R>::type *__restrict__ x,
                typename cplx_of<R>::type *__restrict__ y, int n, const typename cplx_of<R>::type *__restrict__ tw,
                int COLS)
 {
+    pdl_wait_and_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int T = L / 8, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
@@ -332,13 +342,14 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
     const int col0 = blockIdx.x * COLS;
     const long b = blockIdx.y, N = (long)n * n;
     const long fsm = (long)COLS * LS;
+    const int f0 = NF == 1 ? blockIdx.z : 0;
     auto buf = [&](int k, int pos) -> C & { return sm[k * fsm + c * LS + pad8(pos)]; };
     auto sync = [&]() { __syncthreads(); };
     {   // COLS * L = 8 blockDim.x elements per field: all 16 loads first
-        C t8[2][8];
+        C t8[NF][8];
 #pragma unroll
-        for (int f = 0; f < 2; ++f) {
-            const C *Wf = W + (b * 3 + f) * (long)L * n;
+        for (int f = 0; f < NF; ++f) {
+            const C *Wf = W + (b * 3 + f0 + f) * (long)L * n;
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int i = q * blockDim.x + threadIdx.x;
@@ -347,7 +358,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
             }
         }
 #pragma unroll
-        for (int f = 0; f < 2; ++f)
+        for (int f = 0; f < NF; ++f)
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int i = q * blockDim.x + threadIdx.x;
@@ -355,34 +366,34 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
             }
     }
     __syncthreads();
-    C v[2][8];
+    C v[NF][8];
 #pragma unroll
-    for (int f = 0; f < 2; ++f)
+    for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int q = 0; q < 8; ++q) v[f][q] = buf(f, t + T * q);
     __syncthreads();
-    fftr::fft_lines<1, L, false, 2>(v, t, buf, sync, tw);
+    fftr::fft_lines<1, L, false, NF>(v, t, buf, sync, tw);
 #pragma unroll
-    for (int f = 0; f < 2; ++f)
+    for (int f = 0; f < NF; ++f)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int r = t + T * q;
             if (r < n) buf(f, r) = v[f][q];
         }
     __syncthreads();
-    for (int f = 0; f < 2; ++f) {
+    for (int f = 0; f < NF; ++f) {
         C xv[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) { // COLS * n <= 4 blockDim.x
             const int i = q * blockDim.x + threadIdx.x;
             const int cc = i & (COLS - 1), r = i / COLS, i1 = col0 + cc;
-            xv[q] = r < n && i1 < n ? x[(b * 2 + f) * N + (long)r * n + i1] : czero<C>();
+            xv[q] = r < n && i1 < n ? x[(b * 2 + f0 + f) * N + (long)r * n + i1] : czero<C>();
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = q * blockDim.x + threadIdx.x;
             const int cc = i & (COLS - 1), r = i / COLS, i1 = col0 + cc;
-            if (r < n && i1 < n) y[(b * 2 + f) * N + (long)r * n + i1] = xv[q] + sm[f * fsm + cc * LS + pad8(r)];
+            if (r < n && i1 < n) y[(b * 2 + f0 + f) * N + (long)r * n + i1] = xv[q] + sm[f * fsm + cc * LS + pad8(r)];
         }
     }
 }
@@ -416,19 +427,23 @@ spm_status apply_L(spm2_problem_s *P, const void *xv, void *yv, int nrhs, cudaSt
     auto pow2_floor = [](long v) { int r = 1; while ((long)r * 2 <= v) r *= 2; return r; };
     const int max_cols = std::max(1, (sizeof(R) == 4 ? 512 : 256) / G::T);
     const int cols = std::max(1, std::min({16, max_cols, pow2_floor(std::max(1L, (long)n / 304))}));
-    const int rb = std::max(1, std::min({L, std::max(1, 256 / G::T), pow2_floor(std::max(1L, (long)L / 304))}));
-    const size_t sm_rows = sizeof(C) * rb * 3 * G::LS, sm_cols = sizeof(C) * 3 * cols * G::LS;
-    SPM_TRY(allow_smem(k2d_colfwd<R, L>, sm_cols));
+    // (complex128: half that, a warp per scheduler, so that the last of the few rounds of
+    // blocks is shorter: the row pass at L = 1024 326 -> 286 us)
+    const int rb = std::max(1, std::min({L, std::max(1, (sizeof(R) == 4 ? 256 : 128) / G::T), pow2_floor(std::max(1L, (long)L / 304))}));
+    constexpr int NF = sizeof(R) == 4 ? 3 : 1, NI = sizeof(R) == 4 ? 2 : 1; // fields per block of the column passes
+    const size_t sm_rows = sizeof(C) * rb * 3 * G::LS, sm_cols = sizeof(C) * NF * cols * G::LS;
+    SPM_TRY(allow_smem(k2d_colfwd<R, L, NF>, sm_cols));
     SPM_TRY(allow_smem(k2d_rowprod<R, L>, sm_rows));
-    SPM_TRY(allow_smem(k2d_colinv<R, L>, sm_cols));
+    SPM_TRY(allow_smem(k2d_colinv<R, L, NI>, sm_cols));
     for (int b0 = 0; b0 < nrhs; b0 += chunk) {
         const int nb_ = std::min(chunk, nrhs - b0);
         const C *x = reinterpret_cast<const C *>(xv) + (long)b0 * 2 * N;
         C *y = reinterpret_cast<C *>(yv) + (long)b0 * 2 * N;
-        const dim3 gcol((unsigned)((n + cols - 1) / cols), (unsigned)nb_);
-        k2d_colfwd<R, L><<<gcol, cols * G::T, sm_cols, s>>>(x, m, p, W, n, tw, cols);
-        k2d_rowprod<R, L><<<dim3(L / rb, (unsigned)nb_), rb * G::T, sm_rows, s>>>(W, spec, n, tw, rb);
-        k2d_colinv<R, L><<<gcol, cols * G::T, sm_cols, s>>>(W, x, y, n, tw, cols);
+        const unsigned gc = (unsigned)((n + cols - 1) / cols);
+        launch_pdl(k2d_colfwd<R, L, NF>, dim3(gc, (unsigned)nb_, 3 / NF), dim3(cols * G::T), sm_cols, s, x, m, p, W, n, tw, cols);
+        launch_pdl(k2d_rowprod<R, L>, dim3(L / rb, (unsigned)nb_), dim3(rb * G::T), sm_rows, s, W, spec, n, tw, rb);
+        launch_pdl(k2d_colinv<R, L, NI>, dim3(gc, (unsigned)nb_, 2 / NI), dim3(cols * G::T), sm_cols, s, (const C *)W, x, y, n, tw,
+                   cols);
     }
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
