@@ -80,6 +80,19 @@ template <typename R, int L> struct tx_of {
     static constexpr int v = w < L ? w : L; // never wider than a row of L elements
 };
 
+// Blocks per SM asked of the compiler for a strided pass whose threads get at
+// most `regs` registers; 0 leaves its own choice.  Asked for at L = 128 in
+// complex64 only, where that choice is a bad one: k2_cols2 took 74 registers
+// (three blocks; 14.0 us against 12.1 with four), k2_zprod4 100 (still two
+// blocks, its loads in shorter batches; 30.7 us against 26.7 with 128).  One
+// application at n = 64: 70.9 us, 74.1 without.  The other lengths already
+// compile to these numbers, and a bound of one block there makes k2_cols2 keep
+// fewer blocks resident (L = 512: 946 us against 633).
+template <typename R, int L> constexpr int pass_blocks(int regs)
+{
+    return sizeof(R) == 4 && L == 128 ? 65536 / (regs * tx_of<R, L>::v * L / 8) : 0;
+}
+
 constexpr int ZPROD_FOUR = 0, ZPROD_ONE = 1, ZPROD_TMA = 2, ZPROD_E16 = 3, ZPROD_STAGED = 4, ZPROD_SPLIT = 5; // z-pass kernels
 constexpr int ZPLAN_FUSED_XY = 8; // plan bit: x and y passes fused per z-plane (L = 64, 128)
 
@@ -189,7 +202,7 @@ __global__ void __launch_bounds__(tx_of<R, L>::v * L / line_elems(L)) k2_cols(co
 // columns are loaded before either is transformed, and the two transforms share
 // every barrier (fft_lines), so each thread keeps twice the loads in flight.
 template <typename R, int L, int DIR, bool PRUNE>
-__global__ void __launch_bounds__(tx_of<R, L>::v * L / 8) k2_cols2(const typename cplx_of<R>::type *in, typename cplx_of<R>::type *out,
+__global__ void __launch_bounds__(tx_of<R, L>::v * L / 8, pass_blocks<R, L>(64)) k2_cols2(const typename cplx_of<R>::type *in, typename cplx_of<R>::type *out,
                                                                  int nout, long inner, int F, long ib, long if_, long iz, long ob,
                                                                  long of, long oz, const typename cplx_of<R>::type *__restrict__ tw)
 {
@@ -485,7 +498,7 @@ __global__ void __launch_bounds__(256, 2) k2_zsplit(typename cplx_of<R>::type *W
 // zprod, E = 8: the four forward z-transforms run together (shared barriers),
 // then the three products and the three inverse transforms together.
 template <typename R, int L>
-__global__ void __launch_bounds__(tx_of<R, L>::v * L / 8) k2_zprod4(typename cplx_of<R>::type *W2,
+__global__ void __launch_bounds__(tx_of<R, L>::v * L / 8, pass_blocks<R, L>(128)) k2_zprod4(typename cplx_of<R>::type *W2,
                                                                   const typename cplx_of<R>::type *__restrict__ spec,
                                                                   const typename cplx_of<R>::type *__restrict__ tw)
 {
