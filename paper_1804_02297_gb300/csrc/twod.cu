@@ -477,6 +477,8 @@ __device__ __forceinline__ int cls_of(int i1, int i2, int n)
 // (Q v)_{i,c} = sum_{s,d} qtab[cls][c][s][d] v^d_{i+o_s}: one thread per (point, c), all
 // loads before the FMAs.  Complex128 is bound by the FP64 pipe (144 n^2 FMAs: 13 us at
 // n = 239), so blocks are small and evenly placed.
+// The order of the sum (per point s the second field, then the first) is part of the
+// result: 2-D factors magnify the last bit of Q v to 2e-9 of S^-1 Q v on some media.
 constexpr int Q2_THREADS = 64;
 template <typename C>
 __global__ void __launch_bounds__(Q2_THREADS) k2_applyQ(const C *__restrict__ qtab, const C *__restrict__ v,
@@ -503,7 +505,7 @@ __global__ void __launch_bounds__(Q2_THREADS) k2_applyQ(const C *__restrict__ qt
     }
     C acc = czero<C>();
 #pragma unroll
-    for (int s = 0; s < 18; ++s) acc = cfma(a[s], u[s], acc);
+    for (int s = 0; s < 18; s += 2) acc = cfma(a[s], u[s], cfma(a[s + 1], u[s + 1], acc));
     y[(b * 2 + c) * N + i] = acc;
 }
 
