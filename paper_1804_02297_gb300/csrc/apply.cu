@@ -879,10 +879,11 @@ __global__ void __launch_bounds__(256) k2_xinv(const typename cplx_of<R>::type *
 // Half of the L1 for shared memory unless a pass needs more: without a request a pass runs
 // with what the one before it wanted (A complex64, asked for 50 / 75 / 100 %: n = 32 13.2,
 // 13.1, 12.6 us against 14.9; n = 128 438, 460, 514 against 463; n = 256 4077, 4278, 4953
-// against 4114; n = 64 54.2, 56.1, 57.8 against 54.2).
-template <typename K> void allow_smem(K kernel, size_t bytes)
+// against 4114; n = 64 54.2, 56.1, 57.8 against 54.2).  In complex128 the request costs
+// (n = 96 3643 us against 3472, n = 16 50 against 47), so there is none.
+template <typename R, typename K> void allow_smem(K kernel, size_t bytes)
 {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+    if (sizeof(R) == 4) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
     if (bytes > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
@@ -1097,7 +1098,7 @@ spm_status launch_ztma(typename cplx_of<R>::type *W2, const typename cplx_of<R>:
     static int grid_per_sm = 0;
     static int sms = 0;
     if (!grid_per_sm) {
-        allow_smem(k2_ztma<R, L>, smem);
+        allow_smem<R>(k2_ztma<R, L>, smem);
         int dev = 0;
         SPM_CUDA_TRY(cudaGetDevice(&dev));
         SPM_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
@@ -1143,17 +1144,17 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     constexpr size_t sm_zprod4 = 4 * sm_cols;
     static bool attrs = false;
     if (!attrs) {
-        allow_smem(k2_xfwd<R, L, true>, sm_rows);
-        allow_smem(k2_xfwd<R, L, false>, sm_rows);
-        allow_smem(k2_xinv<R, L>, sm_rows);
-        allow_smem(k2_cols<R, L, -1, true>, sm_cols);
-        allow_smem(k2_cols<R, L, 1, false>, sm_cols);
+        allow_smem<R>(k2_xfwd<R, L, true>, sm_rows);
+        allow_smem<R>(k2_xfwd<R, L, false>, sm_rows);
+        allow_smem<R>(k2_xinv<R, L>, sm_rows);
+        allow_smem<R>(k2_cols<R, L, -1, true>, sm_cols);
+        allow_smem<R>(k2_cols<R, L, 1, false>, sm_cols);
         if constexpr (line_elems(L) == 8) {
-            allow_smem(k2_cols2<R, L, -1, true>, 2 * sm_cols);
-            allow_smem(k2_cols2<R, L, 1, false>, 2 * sm_cols);
+            allow_smem<R>(k2_cols2<R, L, -1, true>, 2 * sm_cols);
+            allow_smem<R>(k2_cols2<R, L, 1, false>, 2 * sm_cols);
         }
-        if constexpr (line_elems(L) == 8) allow_smem(k2_zprod4<R, L>, sm_zprod4);
-        allow_smem(k2_zprod1<R, L>, sm_zprod);
+        if constexpr (line_elems(L) == 8) allow_smem<R>(k2_zprod4<R, L>, sm_zprod4);
+        allow_smem<R>(k2_zprod1<R, L>, sm_zprod);
         attrs = true;
     }
     const long n2 = (long)n * n, L2 = (long)L * L;
@@ -1163,8 +1164,8 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
         if (fused) {
             static bool axy = false;
             if (!axy) {
-                allow_smem(k2_xyfwd<R, L>, xyf<R, L>::smem);
-                allow_smem(k2_yxinv<R, L>, xyf<R, L>::smem);
+                allow_smem<R>(k2_xyfwd<R, L>, xyf<R, L>::smem);
+                allow_smem<R>(k2_yxinv<R, L>, xyf<R, L>::smem);
                 axy = true;
             }
             launch_pdl(k2_xyfwd<R, L>, dim3(n, 4, nb), dim3(256), xyf<R, L>::smem, s, xb, m, p, W2, tw);
@@ -1199,7 +1200,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
             constexpr size_t sm16 = zp16<R, L>::smem();
             static bool a16 = false;
             if (!a16) {
-                allow_smem(k3_zpass<R, L>, sm16);
+                allow_smem<R>(k3_zpass<R, L>, sm16);
                 a16 = true;
             }
             launch_pdl(k3_zpass<R, L>, dim3((unsigned)(L2 / zp16<R, L>::TX), nb), dim3(zp16<R, L>::THREADS), sm16, s,
@@ -1212,7 +1213,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
             constexpr size_t smz = zst<R, L>::smem;
             static bool ast = false;
             if (!ast) {
-                allow_smem(k2_zstaged<R, L>, smz);
+                allow_smem<R>(k2_zstaged<R, L>, smz);
                 ast = true;
             }
             launch_pdl(k2_zstaged<R, L>, dim3((unsigned)(L2 / TX), nb), dim3(zst<R, L>::THREADS), smz, s, W2, spec, tw);
@@ -1223,7 +1224,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
         if (!done && zvar == ZPROD_SPLIT) {
             static bool asp = false;
             if (!asp) {
-                allow_smem(k2_zsplit<R, L>, zsp<R, L>::smem);
+                allow_smem<R>(k2_zsplit<R, L>, zsp<R, L>::smem);
                 asp = true;
             }
             launch_pdl(k2_zsplit<R, L>, dim3((unsigned)(L2 / zsp<R, L>::TX), nb), dim3(256), zsp<R, L>::smem, s, W2,
@@ -1753,7 +1754,7 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
     constexpr size_t smem = sizeof(C) * Q_SMEM;
     static bool attr = false;
     if (!attr) {
-        allow_smem(k_q, smem);
+        allow_smem<R>(k_q, smem);
         attr = true;
     }
     launch_pdl(k_q, dim3((unsigned)(face_blocks + edge_blocks + interior_blocks), (unsigned)nrhs), dim3(Q_THREADS),
