@@ -799,7 +799,7 @@ struct NDFactor {
         int ntiles_f, ntiles_b;
     };
     std::vector<Level> levels;
-    int tile_elems = 0, tile_cols = 0; // of the largest tiles
+    int tile_elems = 0, tile_cols = 0; // of the largest tiles (entries rounded up to four)
     bool staged = false;               // tiles copied to shared memory whole
     DevBuf st_tiles, st_bnd, st_rank, st_point; // tiles, boundary unknowns, rank of each point and back
     DenseWork *dense = nullptr; // Gauss-Jordan workspace
@@ -944,6 +944,8 @@ template <typename R> static spm_status build_solve_tiles(NDFactor *F, const std
         cut(at[d], false, lv.tiles_b, lv.ntiles_b);
         F->levels.push_back(lv);
     }
+    // the vectors lie behind a staged tile: whole 16-byte units, also of 4-byte entries
+    F->tile_elems = (F->tile_elems + 3) / 4 * 4;
     auto put = [](DevBuf &buf, const void *src, size_t bytes) -> spm_status {
         SPM_TRY(buf.ensure(std::max<size_t>(bytes, 1)));
         if (bytes) SPM_CUDA_TRY(cudaMemcpy(buf.ptr, src, bytes, cudaMemcpyHostToDevice));
