@@ -1731,8 +1731,8 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
                        qtab, (C *)yv, n);
         } else {
             const dim3 grid((unsigned)((n * n * n + Q_THREADS - 1) / Q_THREADS), 3, (unsigned)nrhs);
-            static const EvenPlacement even(k_q_direct<C, 1>, Q_THREADS);
-            launch_pdl(k_q_direct<C, 1>, grid, dim3(Q_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, (const C *)vv,
+            static PerDevice<EvenPlacement> even;
+            launch_pdl(k_q_direct<C, 1>, grid, dim3(Q_THREADS), even_smem(even, k_q_direct<C, 1>, Q_THREADS, grid), s, (const C *)vv,
                        qtab, (C *)yv, n);
         }
         SPM_CUDA_TRY(cudaGetLastError());

@@ -4,6 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <algorithm>
+#include <map>
+#include <mutex>
+#include <optional>
 #include <string>
 #include <vector>
 
@@ -148,37 +151,61 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// What holds for the device that was current when it was made (a kernel's attributes, what
+// a device can hold), made once for each device, by any thread.  make() gives none when it
+// failed, which is not kept.
+template <typename T> struct PerDevice {
+    std::mutex lock;
+    std::map<int, T> made;
+    template <typename F> std::optional<T> get(F make)
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return std::nullopt;
+        std::lock_guard<std::mutex> hold(lock);
+        const auto at = made.find(dev);
+        if (at != made.end()) return at->second;
+        const std::optional<T> v = make();
+        if (v) made.emplace(dev, *v);
+        return v;
+    }
+};
+
 // Even placement.  A grid that fits the chip at once may be placed unevenly (some SMs
 // full, others idle), which an FP64-bound kernel pays in full: 768 equal blocks of
 // k_q_direct on 152 SMs took 102 us, held to six on an SM 63 us.  smem_for(blocks) is
 // the dynamic shared memory with which at most ceil(blocks / SMs) blocks fit on an SM;
 // zero when the grid takes several waves, whose blocks go where there is room.  Made
-// once per kernel (the queries take microseconds).
+// once per kernel and device (the queries take microseconds).
 struct EvenPlacement {
     int sms = 0, room = 0, most = 0, fixed = 0, per = 0;
-    template <typename K> EvenPlacement(K kernel, int threads)
+    template <typename K> static std::optional<EvenPlacement> of(K kernel, int threads)
     {
+        EvenPlacement e;
         int dev = 0;
         cudaFuncAttributes fa = {};
         if (cudaGetDevice(&dev) != cudaSuccess || cudaFuncGetAttributes(&fa, kernel) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&room, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, 0) != cudaSuccess)
-            per = 0;
-        fixed = 1024 + (int)fa.sharedSizeBytes; // reserved by the system, declared by the kernel
-        if (per > 0 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            most - (int)fa.sharedSizeBytes) != cudaSuccess)
-            per = 0;
+            cudaDeviceGetAttribute(&e.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&e.room, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&e.most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&e.per, kernel, threads, 0) != cudaSuccess ||
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, e.most - (int)fa.sharedSizeBytes) != cudaSuccess)
+            return std::nullopt;
+        e.fixed = 1024 + (int)fa.sharedSizeBytes; // reserved by the system, declared by the kernel
+        return e;
     }
     size_t smem_for(long blocks) const
     {
-        if (per == 0) return 0;
         const long want = (blocks + sms - 1) / sms;
         if (want >= per) return 0;
         return (size_t)std::max(0L, std::min<long>(room / (want + 1) + 1, most + 1024) - fixed); // one more would not fit
     }
 };
+// the same for a kernel's launch on the current device (no padding where its queries fail)
+template <typename K> size_t even_smem(PerDevice<EvenPlacement> &placed, K kernel, int threads, dim3 grid)
+{
+    const std::optional<EvenPlacement> e = placed.get([&] { return EvenPlacement::of(kernel, threads); });
+    return e ? e->smem_for((long)grid.x * grid.y * grid.z) : 0;
+}
 
 // ------------------------------------------------------------ device buffer
 // Owned device allocation: freed by release() or when the owner goes out of

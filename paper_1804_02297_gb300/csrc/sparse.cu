@@ -1403,10 +1403,9 @@ static void each_level(NDFactor *F, KF fwd, KB bwd, L launch)
         if (F->levels[l].ntiles_b > 0) launch(bwd, tiles + F->levels[l].tiles_b, F->levels[l].ntiles_b);
 }
 
-// Opt in to the shared memory (a failure shows as a failed launch), and, where tiles stream
-// through registers, ask for the L1: lines in flight live there, and without a request the
-// SM keeps the division that the kernel before it wanted (S^-1 at n = 32: 314 us among its
-// like, 440 after Q).
+// Opt in to the shared memory, and, where tiles stream through registers, ask for the L1:
+// lines in flight live there, and without a request the SM keeps the division that the
+// kernel before it wanted (S^-1 at n = 32: 314 us among its like, 440 after Q).
 template <typename K> static bool opt_in(K kernel, bool staged, int percent)
 {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024) == cudaSuccess &&
@@ -1418,9 +1417,12 @@ static void launch_levels(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStr
 {
     // percent of 228 KB for the blocks that fit: NB x 256 sums and a reserved kilobyte each
     constexpr int percent = st_blocks<C, NB>() * ((int)sizeof(C) * NB * ST_THREADS + 1024) / 2334 + 1;
-    static const bool allowed = opt_in(k_nd_level<C, S, NB, true, STAGED>, STAGED, percent) &&
-                                opt_in(k_nd_level<C, S, NB, false, STAGED>, STAGED, percent);
-    (void)allowed;
+    static PerDevice<bool> opted;
+    opted.get([]() -> std::optional<bool> { // a failure is the last error, which the solve checks after its launches
+        if (opt_in(k_nd_level<C, S, NB, true, STAGED>, STAGED, percent) && opt_in(k_nd_level<C, S, NB, false, STAGED>, STAGED, percent))
+            return true;
+        return std::nullopt;
+    });
     // at most a 48 KB tile and 32 KB of sums
     const size_t smem = (STAGED ? sizeof(S) * (size_t)F->tile_elems : 0) + sizeof(C) * NB * std::max(ST_THREADS, F->tile_cols);
     each_level(F, k_nd_level<C, S, NB, true, STAGED>, k_nd_level<C, S, NB, false, STAGED>, [&](auto kernel, const SolveTile *t, int n) {

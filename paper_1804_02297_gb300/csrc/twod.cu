@@ -823,9 +823,9 @@ spm_status spm2_apply_A_impl(spm2_problem_s *P, int prec, const void *x, void *y
 template <typename C>
 static void launch_Q2(const C *qtab, const void *v, void *y, int n, int nrhs, cudaStream_t s)
 {
-    static const EvenPlacement even(k2_applyQ<C>, Q2_THREADS);
+    static PerDevice<EvenPlacement> even;
     const dim3 grid(nb((long)n * n, Q2_THREADS), 2, (unsigned)nrhs);
-    launch_pdl(k2_applyQ<C>, grid, dim3(Q2_THREADS), even.smem_for((long)grid.x * grid.y * grid.z), s, qtab,
+    launch_pdl(k2_applyQ<C>, grid, dim3(Q2_THREADS), even_smem(even, k2_applyQ<C>, Q2_THREADS, grid), s, qtab,
                reinterpret_cast<const C *>(v), reinterpret_cast<C *>(y), n);
 }
 

@@ -108,3 +108,22 @@ def test_staged_tiles_leave_the_vectors_aligned(lib, dim, n):
                 staged += 1
         assert staged
     pb.close()
+
+
+def test_a_second_device_is_opted_in(lib):
+    """What a kernel is allowed holds for one device: Q's padding for even placement and the
+    solve's tiles with their sums are asked for on every device that launches them."""
+    for dev in (0, 1):
+        lib.fake_device(dev)
+        for dim, n in ((2, 64), (3, 16)):
+            pb = Prob(lib, dim, n)
+            assert pb.call("apply_Q", pb.h, C128, P(256), P(1 << 40), 1, None) == 0
+            for prec in (C128, C64):
+                assert pb.call("factor_S", pb.h, prec) == 0
+                for nrhs in (1, 2, 4, 8, 16):
+                    assert pb.solve(prec, nrhs) == 0
+            pb.close()
+        seen = launches(lib)
+        assert all(d == dev and k != "-" for d, _, _, k in seen)
+        assert max(s for _, s, _, k in seen if "k_nd_level" in k) > 48 * 1024
+        assert max(s for _, s, _, k in seen if "k2_applyQ" in k) > 48 * 1024
