@@ -121,6 +121,7 @@ struct BatchFront {
 };
 
 constexpr int BP_NB = 8, BP_THREADS = 256;
+constexpr int BATCH_LINES[] = {1536, 1024, 512}; // unknowns of the largest fronts batched
 template <typename C> struct BatchPanel {
     C prow[BP_NB][BP_NB];               // scaled pivot row of each step ([jj][jj]: 1 / pivot)
     int nmove;                          // rows the panel's swaps gave new contents
@@ -780,6 +781,7 @@ __global__ void k_to_half(__half2 *dst, const float2 *__restrict__ src, int m, i
 struct NDFactor {
     int prec = 0;
     int variant = 0;         // nested-dissection tree variant (cut offsets)
+    int batch_line = 0;      // unknowns up to which fronts were batched
     int raised_pivots = 0;   // pivots raised by the static perturbation
     size_t stored_bytes = 0; // bytes of the stored blocks (G and X, plus half-storage scales)
     bool half_store = false; // blocks as scaled binary16 pairs (complex64 factor only)
@@ -1010,7 +1012,7 @@ static spm_status factor_panels(const BatchFront *fronts, int count, int fm, int
 }
 
 template <typename R>
-static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store, int variant)
+static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store, int variant, int most)
 {
     using C = typename cplx_of<R>::type;
     const int n1 = SY.dims[0], n2 = SY.dims[1], n3d = SY.dims[2], D = SY.D;
@@ -1109,8 +1111,9 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
     // per-front path rounds differently, and 2-D factors have near-singular boxes often
     // enough (one medium in ten at n = 239) that S^-1 moves by more than 1e-9.
     std::vector<char> batched(NN, 0);
-    for (const int fmax : {1536, 1024, 512}) {
-        if (n3d == 1 && fmax > 512) continue;
+    for (const int fmax : BATCH_LINES) {
+        if (fmax > (n3d == 1 ? 512 : most)) continue;
+        F->batch_line = fmax;
         double bytes = 0;
         for (int id = 0; id < NN; ++id) { // postorder: children before parents
             const Node &nd = nodes[id];
@@ -1559,10 +1562,22 @@ spm_status factor_once(const SparseSys &SY, int prec, int variant, NDFactor *&sl
 {
     spm_factor_free(slot);
     slot = nullptr;
-    NDFactor *F = new NDFactor();
-    F->prec = prec == SPM_C128 ? SPM_C128 : SPM_C64;
-    spm_status st = prec == SPM_C128 ? factor_typed<double>(SY, F, false, variant)
-                                     : factor_typed<float>(SY, F, prec == SPM_C64H, variant);
+    // A higher line takes more memory (3-D complex128 n = 32: 9.8 GB at the most with 1536,
+    // 7.9 with 512): where it ends, the next lower line is tried.
+    NDFactor *F = nullptr;
+    spm_status st = SPM_ERR_OOM;
+    int most = BATCH_LINES[0];
+    while (st == SPM_ERR_OOM && most > 0) {
+        if (F) cudaGetLastError(); // of the allocation that failed
+        delete F;
+        F = new NDFactor();
+        F->prec = prec == SPM_C128 ? SPM_C128 : SPM_C64;
+        st = prec == SPM_C128 ? factor_typed<double>(SY, F, false, variant, most)
+                              : factor_typed<float>(SY, F, prec == SPM_C64H, variant, most);
+        most = 0;
+        for (const int line : BATCH_LINES)
+            if (line < F->batch_line && !F->half_store) most = std::max(most, line);
+    }
     if (st != SPM_OK) {
         delete F;
         return st;

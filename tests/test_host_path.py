@@ -127,3 +127,19 @@ def test_a_second_device_is_opted_in(lib):
         assert all(d == dev and k != "-" for d, _, _, k in seen)
         assert max(s for _, s, _, k in seen if "k_nd_level" in k) > 48 * 1024
         assert max(s for _, s, _, k in seen if "k2_applyQ" in k) > 48 * 1024
+
+
+def test_factor_takes_less_where_memory_ends(lib):
+    """3-D n = 32 in complex128: fronts of up to 1536 unknowns advance together, which takes
+    a quarter more memory than a line at 512; where that is not there, the lower lines are
+    tried before the factor is refused."""
+    pb = Prob(lib, 3, 32)
+    lib.fake_peak()
+    assert pb.call("factor_S", pb.h, C128) == 0
+    need = lib.fake_peak()
+    pb.close()
+    pb = Prob(lib, 3, 32)
+    for share, status in ((0.9, 0), (0.5, 3), (1.0, 0)):
+        lib.fake_capacity(int(share * need))
+        assert pb.call("factor_S", pb.h, C128) == status
+    pb.close()
