@@ -474,39 +474,50 @@ __device__ __forceinline__ int cls_of(int i1, int i2, int n)
     return c1 + 3 * c2;
 }
 
-// (Q v)_{i,c} = sum_{s,d} qtab[cls][c][s][d] v^d_{i+o_s}: one thread per (point, c), all
-// loads before the FMAs.  Complex128 is bound by the FP64 pipe (144 n^2 FMAs: 13 us at
-// n = 239), so blocks are small and evenly placed.
+// (Q v)_{i,c} = sum_{s,d} qtab[cls][c][s][d] v^d_{i+o_s}, all loads of a thread before its
+// FMAs.  NC = 1: one thread per (point, c); complex128 is bound by the FP64 pipe (144 n^2
+// FMAs: 13 us at n = 239), so blocks are small and evenly placed.  NC = 2: one thread per
+// point for both c, in complex64, whose FMAs are nothing beside the loads (n = 1024 34.4 us
+// with NC = 1 and 16.1 with 2, eight fields at n = 479 59 and 26.2).  Points are counted
+// through all right-hand sides, so that small grids fill their blocks too.
 // The order of the sum (per point s the second field, then the first) is part of the
 // result: 2-D factors magnify the last bit of Q v to 2e-9 of S^-1 Q v on some media.
-constexpr int Q2_THREADS = 64;
+template <typename C> struct Q2Shape {
+    static constexpr int NC = sizeof(C) == 16 ? 1 : 2, THREADS = sizeof(C) == 16 ? 64 : 256;
+};
 template <typename C>
-__global__ void __launch_bounds__(Q2_THREADS) k2_applyQ(const C *__restrict__ qtab, const C *__restrict__ v,
-                                                        C *__restrict__ y, int n)
+__global__ void __launch_bounds__(Q2Shape<C>::THREADS) k2_applyQ(const C *__restrict__ qtab, const C *__restrict__ v,
+                                                             C *__restrict__ y, int n, long total)
 {
     pdl_wait_and_trigger();
-    const long N = (long)n * n, i = (long)blockIdx.x * Q2_THREADS + threadIdx.x;
-    const int c = blockIdx.y;
-    const long b = blockIdx.z;
-    if (i >= N) return;
-    const int i1 = (int)(i % n), i2 = (int)(i / n);
-    const C *q = qtab + (cls_of(i1, i2, n) * 2 + c) * 18, *vb = v + b * 2 * N + i;
-    C a[18], u[18];
+    constexpr int NC = Q2Shape<C>::NC;
+    const long gid = (long)blockIdx.x * Q2Shape<C>::THREADS + threadIdx.x;
+    if (gid >= total) return;
+    const long N = (long)n * n;
+    // (64-bit divisions are 2 us at the start of every thread)
+    const long b = total <= 0x7fffffffL ? (long)((unsigned)gid / (unsigned)N) : gid / N, i = gid - b * N;
+    const int c0 = NC == 1 ? (int)blockIdx.y : 0, i1 = (int)i % n, i2 = (int)i / n;
+    const C *q = qtab + (cls_of(i1, i2, n) * 2 + c0) * 18, *vb = v + b * 2 * N + i;
+    C a[NC][18], u[18];
 #pragma unroll
     for (int s = 0; s < 9; ++s) {
         const int o1 = s % 3 - 1, o2 = s / 3 - 1;
         const bool in = i1 + o1 >= 0 && i1 + o1 < n && i2 + o2 >= 0 && i2 + o2 < n;
 #pragma unroll
         for (int d = 0; d < 2; ++d) {
-            a[2 * s + d] = q[2 * s + d];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) a[c][2 * s + d] = q[18 * c + 2 * s + d];
             u[2 * s + d] = czero<C>();
             if (in) u[2 * s + d] = vb[d * N + (long)o2 * n + o1];
         }
     }
-    C acc = czero<C>();
 #pragma unroll
-    for (int s = 0; s < 18; s += 2) acc = cfma(a[s], u[s], cfma(a[s + 1], u[s + 1], acc));
-    y[(b * 2 + c) * N + i] = acc;
+    for (int c = 0; c < NC; ++c) {
+        C acc = czero<C>();
+#pragma unroll
+        for (int s = 0; s < 18; s += 2) acc = cfma(a[c][s], u[s], cfma(a[c][s + 1], u[s + 1], acc));
+        y[(b * 2 + c0 + c) * N + i] = acc;
+    }
 }
 
 // S[i][s][c][f] = alpha[(f,o),c] + beta[(f,o),c] m_j + beta[(2,o),c] p^f_j, j = i + o_s
@@ -823,10 +834,15 @@ spm_status spm2_apply_A_impl(spm2_problem_s *P, int prec, const void *x, void *y
 template <typename C>
 static void launch_Q2(const C *qtab, const void *v, void *y, int n, int nrhs, cudaStream_t s)
 {
-    static PerDevice<EvenPlacement> even;
-    const dim3 grid(nb((long)n * n, Q2_THREADS), 2, (unsigned)nrhs);
-    launch_pdl(k2_applyQ<C>, grid, dim3(Q2_THREADS), even_smem(even, k2_applyQ<C>, Q2_THREADS, grid), s, qtab,
-               reinterpret_cast<const C *>(v), reinterpret_cast<C *>(y), n);
+    constexpr int T = Q2Shape<C>::THREADS;
+    const long total = (long)n * n * nrhs;
+    const dim3 grid(nb(total, T), 2 / Q2Shape<C>::NC);
+    size_t pad = 0;
+    if constexpr (sizeof(C) == 16) {
+        static PerDevice<EvenPlacement> even;
+        pad = even_smem(even, k2_applyQ<C>, T, grid);
+    }
+    launch_pdl(k2_applyQ<C>, grid, dim3(T), pad, s, qtab, reinterpret_cast<const C *>(v), reinterpret_cast<C *>(y), n, total);
 }
 
 spm_status spm2_apply_Q_impl(spm2_problem_s *P, int prec, const void *v, void *y, int nrhs, cudaStream_t s)

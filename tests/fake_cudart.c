@@ -34,13 +34,13 @@ void fake_capacity(size_t bytes) { capacity = bytes; }
 size_t fake_used(void) { return used; }
 size_t fake_peak(void) { size_t p = peak; peak = used; return p; }
 /* one line per launch through the extended interface: device, shared memory, int argument
- * (k_nd_level: the entries of a staged tile), kernel; a line "-" for every refused one */
+ * (k_nd_level: the entries of a staged tile), threads, kernel ("-" where refused) */
 const char *fake_log(void) { return text ? text : ""; }
 void fake_clear(void) { text_len = 0; if (text) text[0] = 0; }
-static void say(int d, size_t smem, int arg, const char *name)
+static void say(int d, size_t smem, int arg, long threads, const char *name)
 {
     if (text_cap - text_len < 400) text = realloc(text, text_cap = 2 * text_cap + 4096);
-    text_len += (size_t)sprintf(text + text_len, "%d %zu %d %s\n", d, smem, arg, name);
+    text_len += (size_t)sprintf(text + text_len, "%d %zu %d %ld %s\n", d, smem, arg, threads, name);
 }
 
 void **__cudaRegisterFatBinary(void *b) { return (void **)b; }
@@ -63,20 +63,21 @@ unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, cudaStream_t s
 cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *smem, void *s)
 { *g = call.g; *b = call.b; *smem = call.smem; *(cudaStream_t *)s = call.s; return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
-static cudaError_t launch(const void *f, size_t smem, void **args, int log)
+static cudaError_t launch(const void *f, dim3 g, dim3 b, size_t smem, void **args, int log)
 {
     const int i = find(f);
+    const long threads = (long)g.x * g.y * g.z * b.x * b.y * b.z;
     if (i < 0) return fail(cudaErrorInvalidDeviceFunction);
     const int arg = strstr(funcs[i].name, "k_nd_level") ? *(int *)args[7] : 0;
-    if (smem > (size_t)funcs[i].smem[device]) { say(device, smem, arg, "-"); return fail(cudaErrorInvalidValue); }
-    if (log) say(device, smem, arg, funcs[i].name);
+    if (smem > (size_t)funcs[i].smem[device]) { say(device, smem, arg, threads, "-"); return fail(cudaErrorInvalidValue); }
+    if (log) say(device, smem, arg, threads, funcs[i].name);
     return cudaSuccess;
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t s)
-{ (void)g; (void)b; (void)s; return launch((const void *)k, smem, args, 0); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) { return launch(f, c->dynamicSmemBytes, args, 1); }
+{ (void)s; return launch((const void *)k, g, b, smem, args, 0); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) { return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, args, 1); }
 cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t s)
-{ (void)g; (void)b; (void)s; return launch(f, smem, args, 0); }
+{ (void)s; return launch(f, g, b, smem, args, 0); }
 cudaError_t cudaFuncSetAttribute(const void *f, enum cudaFuncAttribute a, int v)
 {
     const int i = find(f);

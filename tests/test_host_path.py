@@ -79,10 +79,10 @@ class Prob:
 
 
 def launches(lib):
-    """(device, shared bytes, argument, kernel) of every launch since the last clear."""
-    out = [line.split(" ", 3) for line in lib.fake_log().decode().splitlines()]
+    """(device, shared bytes, argument, threads, kernel) of every launch since the last clear."""
+    out = [line.split(" ", 4) for line in lib.fake_log().decode().splitlines()]
     lib.fake_clear()
-    return [(int(d), int(s), int(a), k) for d, s, a, k in out]
+    return [(int(d), int(s), int(a), int(t), k) for d, s, a, t, k in out]
 
 
 @pytest.mark.parametrize("dim,n", [(2, 23), (2, 243), (2, 246), (3, 16)])
@@ -97,7 +97,7 @@ def test_staged_tiles_leave_the_vectors_aligned(lib, dim, n):
         staged = 0
         for nrhs in (1, 2, 3, 4, 5, 16):
             assert pb.solve(C64 if prec == C64H else prec, nrhs) == 0
-            for _, smem, tile, kernel in launches(lib):
+            for _, smem, tile, _, kernel in launches(lib):
                 m = re.search(r"k_nd_levelI(6float2|7double2)(S\d?_|7__half2)Li(\d+)ELb\dELb(\d)E", kernel)
                 if not m or m.group(4) == "0":
                     continue
@@ -124,9 +124,9 @@ def test_a_second_device_is_opted_in(lib):
                     assert pb.solve(prec, nrhs) == 0
             pb.close()
         seen = launches(lib)
-        assert all(d == dev and k != "-" for d, _, _, k in seen)
-        assert max(s for _, s, _, k in seen if "k_nd_level" in k) > 48 * 1024
-        assert max(s for _, s, _, k in seen if "k2_applyQ" in k) > 48 * 1024
+        assert all(d == dev and k != "-" for d, _, _, _, k in seen)
+        assert max(s for _, s, _, _, k in seen if "k_nd_level" in k) > 48 * 1024
+        assert max(s for _, s, _, _, k in seen if "k2_applyQ" in k) > 48 * 1024
 
 
 def test_factor_takes_less_where_memory_ends(lib):
@@ -142,4 +142,19 @@ def test_factor_takes_less_where_memory_ends(lib):
     for share, status in ((0.9, 0), (0.5, 3), (1.0, 0)):
         lib.fake_capacity(int(share * need))
         assert pb.call("factor_S", pb.h, C128) == status
+    pb.close()
+
+
+@pytest.mark.parametrize("n,nrhs", [(4, 1), (4, 4000), (5, 7), (119, 64), (479, 8)])
+def test_2d_q_threads(lib, n, nrhs):
+    """2-D Q reads a point's neighbours once in complex64 (a thread per point; a thread per
+    component took 1.5 times as long at eight fields of n = 479), twice in complex128, and
+    leaves no block partly empty but the last."""
+    pb = Prob(lib, 2, n)
+    for prec, each, block in ((C64, 1, 256), (C128, 2, 64)):
+        launches(lib)
+        assert pb.call("apply_Q", pb.h, prec, P(256), P(1 << 40), nrhs, None) == 0
+        (_, _, _, threads, kernel), = launches(lib)
+        assert "k2_applyQ" in kernel
+        assert threads == each * -(-n * n * nrhs // block) * block
     pb.close()
