@@ -127,10 +127,12 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 // (griddepcontrol.wait) for the previous grid to complete and its memory to be
 // visible before their first global access.  Launched without the attribute,
 // both instructions are no-ops.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_and_trigger()
 {
-    asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    pdl_wait();
+    pdl_trigger();
 }
 
 // A failed launch sets the runtime's last error, which every apply checks after

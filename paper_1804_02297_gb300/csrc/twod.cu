@@ -175,6 +175,24 @@ template <int L> struct Geo2 {
     static constexpr int LS = L + L / 8; // padded line stride
 };
 
+// When a pass lets the blocks of the next one be placed.  A grid that leaves the chip room
+// and does so at its start has the next pass's blocks placed beside its own, where the room
+// is and not evenly, and the pass that they make up lasts as long as the SM with the most
+// of them (complex64, n = 300 51.1 us against 43.6 without programmatic launches, eight
+// fields at n = 119 31.4 against 27.1).  Such a pass triggers before its last stores (38.0,
+// 21.9 us), which still hides the launch.  At its start triggers a pass of so few warps
+// that where they are makes no difference (ten on an SM in complex64: n = 239 16.4 us
+// against 17.6; five in complex128, whose instructions hold a scheduler for 64 cycles:
+// three fields at n = 64 45.9 against 47.9), or of so many that the chip is full until its
+// last blocks (16 of 64 on an SM are resident), which at L = 2048 is every one (complex64,
+// two fields at n = 959 346 us against 350).
+template <typename R, int L> __device__ __forceinline__ bool trigger_early()
+{
+    if constexpr (L >= 2048) return true;
+    const long warps = (long)gridDim.x * gridDim.y * gridDim.z * ((blockDim.x + 31) / 32);
+    return warps <= (sizeof(R) == 4 ? 10 : 5) * 152 || warps >= 64 * 152;
+}
+
 // Pass 1, one column i1 < n per line, COLS adjacent columns per block: the
 // weights w = [m x^1, m x^2, p.x] of the block's columns staged in shared
 // memory (coalesced across columns), the three fields transformed along x2
@@ -190,7 +208,8 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
                const typename cplx_of<R>::type *__restrict__ p, typename cplx_of<R>::type *__restrict__ W, int n,
                const typename cplx_of<R>::type *__restrict__ tw, int COLS)
 {
-    pdl_wait_and_trigger();
+    pdl_wait();
+    if (trigger_early<R, L>()) pdl_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int T = L / 8, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
@@ -253,6 +272,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
 #pragma unroll
         for (int q = 0; q < 8; ++q) buf(f, t + T * q) = v[f][q];
     __syncthreads();
+    if constexpr (L < 2048) pdl_trigger(); // again is nothing
     for (int f = 0; f < NF; ++f) {
         C *Wf = W + (b * 3 + f0 + f) * (long)L * n;
 #pragma unroll
@@ -274,7 +294,8 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k2d_rowprod(typen
                                                    const typename cplx_of<R>::type *__restrict__ spec, int n,
                                                    const typename cplx_of<R>::type *__restrict__ tw, int RB)
 {
-    pdl_wait_and_trigger();
+    pdl_wait();
+    if (trigger_early<R, L>()) pdl_trigger();
     using C = typename cplx_of<R>::type;
     using G = Geo2<L>;
     constexpr int T = G::T, H = L / 2 + 1;
@@ -314,6 +335,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k2d_rowprod(typen
         y[1][q] = cfma(k0, v[1][q], cmul(k2, v[2][q]));
     }
     fftr::fft_lines<1, L, false, 2>(y, t, buf, sync, tw);
+    if constexpr (L < 2048) pdl_trigger(); // again is nothing
 #pragma unroll
     for (int f = 0; f < 2; ++f)
 #pragma unroll
@@ -333,7 +355,8 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
                typename cplx_of<R>::type *__restrict__ y, int n, const typename cplx_of<R>::type *__restrict__ tw,
                int COLS)
 {
-    pdl_wait_and_trigger();
+    pdl_wait();
+    if (trigger_early<R, L>()) pdl_trigger();
     using C = typename cplx_of<R>::type;
     constexpr int T = L / 8, LS = L + L / 8;
     extern __shared__ unsigned char smem_raw[];
@@ -381,6 +404,7 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 512 : 256)
             if (r < n) buf(f, r) = v[f][q];
         }
     __syncthreads();
+    if constexpr (L < 2048) pdl_trigger(); // again is nothing
     for (int f = 0; f < NF; ++f) {
         C xv[4];
 #pragma unroll
