@@ -229,8 +229,8 @@ spm_status spm_solve_S(spm_problem prob, spm_prec prec, const void *b_dev, void 
 /* Apply plan (process-wide, per FFT length L = 2n or the radix-3 lengths 96
  * and 192, and per apply precision SPM_C128 / SPM_C64): the z-pass kernel.
  *   0  four lines per thread block with all fields in registers (lengths other
- *      than 96 and 192; up to L = 32 a group of threads per field, the fields
- *      meeting in shared memory),
+ *      than 96 and 192; at L <= 16, and 32 in complex128, a group of threads per
+ *      field, the fields meeting in shared memory),
  *   1  one field at a time after a cp.async prefetch of all four (L >= 32, 96, 192),
  *   2  persistent, fed by TMA bulk-tensor copies into two shared-memory stages
  *      (L >= 32),

@@ -547,15 +547,19 @@ __global__ void __launch_bounds__(tx_of<R, L>::v * L / 8, pass_blocks<R, L>(128)
         for (int q = 0; q < 4; ++q) base[d * fs + (long)(t + T * q) * L2] = v[d][q];
 }
 
-// The same on small grids (L <= 32), a line per thread group: a quarter of the block's
-// threads per field, TX adjacent columns.  The groups transform their fields side by side,
-// a warp each; p.E's transform goes to the other three through shared
-// memory; they form the product and transform back.  Four times the warps, each with two
-// transforms instead of seven one after another: in complex128 a warp's FP64 instruction
-// takes 64 cycles, and at n = 16 the four-line kernel is 128 warps on 608 schedulers
-// (33.9 us; this one 14.3; n = 8 28.7 and 12.3; complex64 6.8 and 5.8).  From L = 64 on the
-// four-line kernel has warps enough and shares its twiddles and spectra between the
-// fields (complex64 n = 64: 30.7 against 45.1 us, complex128 567 against 590).
+// The same on small grids, a line per thread group: a quarter of the block's threads per
+// field, TX adjacent columns.  The groups transform their fields side by side, a warp each;
+// p.E's transform goes to the other three through shared memory; they form the product and
+// transform back.  Four times the warps, each with two transforms instead of seven one after
+// another: in complex128 a warp's FP64 instruction takes 64 cycles, and at n = 16 the
+// four-line kernel is 128 warps on 608 schedulers (33.9 us; this one 14.3; n = 8 28.7 and
+// 12.3).  It serves complex128 up to L = 32 and complex64 up to 16; at L = 32 in complex64
+// the four-line kernel, which shares its twiddles and spectra between the fields, is little
+// slower for one right-hand side (6.8 us against 5.8) and faster for blocks of them (A with
+// 8 16.9 us against 18.0, with 64 39.7 against 49.8), as it is from L = 64 on in both
+// (complex64 n = 64: 30.7 against 45.1 us, complex128 567 against 590).  By L alone, so that
+// a block of right-hand sides gives the bits of single ones.
+template <typename R, int L> constexpr bool zfield_serves() { return L <= (sizeof(R) == 8 ? 32 : 16); }
 template <typename R, int L> struct zfl {
     using C = typename cplx_of<R>::type;
     static constexpr int T = L / 8;
@@ -1153,7 +1157,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
             allow_smem<R>(k2_cols2<R, L, -1, true>, 2 * sm_cols);
             allow_smem<R>(k2_cols2<R, L, 1, false>, 2 * sm_cols);
         }
-        if constexpr (line_elems(L) == 8) allow_smem<R>(k2_zprod4<R, L>, sm_zprod4);
+        if constexpr (line_elems(L) == 8 && !zfield_serves<R, L>()) allow_smem<R>(k2_zprod4<R, L>, sm_zprod4);
         allow_smem<R>(k2_zprod1<R, L>, sm_zprod);
         attrs = true;
     }
@@ -1234,7 +1238,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     }
     if constexpr (line_elems(L) == 8) {
         if (!done && zvar == ZPROD_FOUR) {
-            if constexpr (L <= 32)
+            if constexpr (zfield_serves<R, L>())
                 launch_pdl(k2_zfield<R, L>, dim3((unsigned)(L2 / zfl<R, L>::TX), nb), dim3(zfl<R, L>::THREADS), zfl<R, L>::smem,
                            s, W2, spec, tw);
             else

@@ -40,7 +40,7 @@ def lib(tmp_path_factory):
     lib.fake_capacity.argtypes = [ctypes.c_size_t]
     lib.spm_create_problem.argtypes = [ctypes.c_int, ctypes.c_double, P, P, ctypes.c_int, P, P]
     lib.spm2_create_problem.argtypes = lib.spm_create_problem.argtypes
-    for name in ("set_stencils", "factor_S", "apply_Q", "solve_S", "destroy"):
+    for name in ("set_stencils", "factor_S", "apply_A", "apply_Q", "solve_S", "destroy"):
         for p in ("spm_", "spm2_"):
             f = getattr(lib, p + name)
             f.argtypes = {"set_stencils": [P, P, P], "factor_S": [P, ctypes.c_int], "destroy": [P]}.get(
@@ -157,4 +157,19 @@ def test_2d_q_threads(lib, n, nrhs):
         (_, _, _, threads, kernel), = launches(lib)
         assert "k2_applyQ" in kernel
         assert threads == each * -(-n * n * nrhs // block) * block
+    pb.close()
+
+
+@pytest.mark.parametrize("n,prec,kernel", [(8, C64, "k2_zfield"), (16, C64, "k2_zprod4"), (32, C64, "k2_zprod4"),
+                                           (8, C128, "k2_zfield"), (16, C128, "k2_zfield"), (32, C128, "k2_zprod4")])
+def test_z_pass_of_plan_0(lib, n, prec, kernel):
+    """A warp per field where the four-line kernel leaves the schedulers idle: not at L = 32
+    in complex64 (64 fields 49.8 us against 39.7).  By L alone, whatever the block."""
+    pb = Prob(lib, 3, n)
+    assert lib.spm_set_apply_plan(prec, 2 * n, 0) == 0
+    for nrhs in (1, 64):
+        launches(lib)
+        assert pb.call("apply_A", pb.h, prec, P(256), P(1 << 40), nrhs, None) == 0
+        z = {m for *_, k in launches(lib) for m in ("k2_zfield", "k2_zprod4", "k2_zprod1") if m in k}
+        assert z == {kernel}
     pb.close()
