@@ -136,21 +136,29 @@ __device__ __forceinline__ void pdl_wait_and_trigger()
 }
 
 // A failed launch sets the runtime's last error, which every apply checks after
-// its launches (cudaGetLastError), as for <<<>>> launches.
+// its launches (cudaGetLastError), as for <<<>>> launches.  shared >= 0 asks for that
+// percentage of the L1 as shared memory, for this launch.
 template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+void launch_pdl_l1(int shared, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
 {
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = (unsigned)shared;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = shared >= 0 ? 2 : 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+template <typename... KArgs, typename... Args>
+void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args)
+{
+    launch_pdl_l1(-1, kernel, grid, block, smem, s, args...);
 }
 
 // What holds for the device that was current when it was made (a kernel's attributes, what

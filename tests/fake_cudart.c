@@ -33,8 +33,9 @@ void fake_device(int d) { device = d; }
 void fake_capacity(size_t bytes) { capacity = bytes; }
 size_t fake_used(void) { return used; }
 size_t fake_peak(void) { size_t p = peak; peak = used; return p; }
-/* one line per launch through the extended interface: device, shared memory, int argument
- * (k_nd_level: the entries of a staged tile), threads, kernel ("-" where refused) */
+/* one line per launch through the extended interface: device, shared memory, a number
+ * (k_nd_level: the entries of a staged tile; others: the share of the L1 that the launch asks
+ * for, 0 if none), threads, kernel ("-" where refused) */
 const char *fake_log(void) { return text ? text : ""; }
 void fake_clear(void) { text_len = 0; if (text) text[0] = 0; }
 static void say(int d, size_t smem, int arg, long threads, const char *name)
@@ -63,21 +64,27 @@ unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t smem, cudaStream_t s
 cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *smem, void *s)
 { *g = call.g; *b = call.b; *smem = call.smem; *(cudaStream_t *)s = call.s; return cudaSuccess; }
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
-static cudaError_t launch(const void *f, dim3 g, dim3 b, size_t smem, void **args, int log)
+static cudaError_t launch(const void *f, dim3 g, dim3 b, size_t smem, void **args, int shared, int log)
 {
     const int i = find(f);
     const long threads = (long)g.x * g.y * g.z * b.x * b.y * b.z;
     if (i < 0) return fail(cudaErrorInvalidDeviceFunction);
-    const int arg = strstr(funcs[i].name, "k_nd_level") ? *(int *)args[7] : 0;
+    const int arg = strstr(funcs[i].name, "k_nd_level") ? *(int *)args[7] : shared;
     if (smem > (size_t)funcs[i].smem[device]) { say(device, smem, arg, threads, "-"); return fail(cudaErrorInvalidValue); }
     if (log) say(device, smem, arg, threads, funcs[i].name);
     return cudaSuccess;
 }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t s)
-{ (void)s; return launch((const void *)k, g, b, smem, args, 0); }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) { return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, args, 1); }
+{ (void)s; return launch((const void *)k, g, b, smem, args, 0, 0); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args)
+{
+    int shared = 0;
+    for (unsigned i = 0; i < c->numAttrs; ++i)
+        if (c->attrs[i].id == cudaLaunchAttributePreferredSharedMemoryCarveout) shared = (int)c->attrs[i].val.sharedMemCarveout;
+    return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, args, shared, 1);
+}
 cudaError_t cudaLaunchCooperativeKernel(const void *f, dim3 g, dim3 b, void **args, size_t smem, cudaStream_t s)
-{ (void)s; return launch(f, g, b, smem, args, 0); }
+{ (void)s; return launch(f, g, b, smem, args, 0, 0); }
 cudaError_t cudaFuncSetAttribute(const void *f, enum cudaFuncAttribute a, int v)
 {
     const int i = find(f);

@@ -79,7 +79,7 @@ class Prob:
 
 
 def launches(lib):
-    """(device, shared bytes, argument, threads, kernel) of every launch since the last clear."""
+    """(device, shared bytes, number, threads, kernel) of every launch since the last clear."""
     out = [line.split(" ", 4) for line in lib.fake_log().decode().splitlines()]
     lib.fake_clear()
     return [(int(d), int(s), int(a), int(t), k) for d, s, a, t, k in out]
@@ -172,4 +172,16 @@ def test_z_pass_of_plan_0(lib, n, prec, kernel):
         assert pb.call("apply_A", pb.h, prec, P(256), P(1 << 40), nrhs, None) == 0
         z = {m for *_, k in launches(lib) for m in ("k2_zfield", "k2_zprod4", "k2_zprod1") if m in k}
         assert z == {kernel}
+    pb.close()
+
+
+@pytest.mark.parametrize("n,nrhs,half", [(4, 1, True), (16, 8, True), (16, 64, False), (64, 1, True), (64, 8, False), (96, 1, False)])
+def test_3d_q_asks_for_half_of_the_l1_on_few_blocks(lib, n, nrhs, half):
+    """Complex64 Q: many blocks need more of the L1 as shared memory than half (16 fields at
+    n = 64 225 us against 212)."""
+    pb = Prob(lib, 3, n)
+    launches(lib)
+    assert pb.call("apply_Q", pb.h, C64, P(256), P(1 << 40), nrhs, None) == 0
+    (_, _, shared, _, kernel), = launches(lib)
+    assert "k_q" in kernel and shared == (50 if half else 0)
     pb.close()
