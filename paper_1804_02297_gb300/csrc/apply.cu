@@ -1760,10 +1760,10 @@ spm_status apply_Q_typed(spm_problem_s *P, const void *vv, void *yv, int nrhs, c
     const dim3 grid((unsigned)(face_blocks + edge_blocks + interior_blocks), (unsigned)nrhs);
     // Half of the L1 for shared memory, as the passes before it, while the blocks are few:
     // three on an SM, and no change of the division in between (Q A n = 32 19.1 us against
-    // 21.8, n = 48 51 against 61, n = 64 70.5 against 78).  From about 2000 blocks on more
+    // 21.8, n = 48 51 against 61, n = 64 70.5 against 78).  From about 2400 blocks on more
     // of them on an SM count (Q n = 96 45.6 us against 46.8, 16 fields at n = 64 212
     // against 225, 64 at n = 16 48.9 against 52.1).
-    const int shared = (long)grid.x * grid.y <= 13 * 152 ? 50 : -1;
+    const int shared = (long)grid.x * grid.y <= 16 * 152 ? 50 : -1;
     launch_pdl_l1(shared, k_q, grid, dim3(Q_THREADS), smem, s, v, qa, qtab, y, n, face_blocks, edge_blocks, nedge);
     SPM_CUDA_TRY(cudaGetLastError());
     return SPM_OK;
