@@ -1133,6 +1133,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     constexpr int n = L / 2, T = L / line_elems(L), TX = tx_of<R, L>::v;
     constexpr int LPB = 256 / T > 0 ? 256 / T : 1;
     constexpr size_t sm_rows = sizeof(C) * LPB * (L + L / 8), sm_cols = sizeof(C) * L * TX;
+    constexpr bool APART = (long)n * n * T < 32 * 4 * 152; // one field's rows may be that few
     // rows per block: 256 threads, fewer (down to a warp) while that leaves under two
     // blocks for each of 152 SMs: x-forward at n = 16 in complex128 was 4 blocks and
     // 40 us, with 32 it takes 21
@@ -1148,7 +1149,7 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
     constexpr size_t sm_zprod4 = 4 * sm_cols;
     static bool attrs = false;
     if (!attrs) {
-        allow_smem<R>(k2_xfwd<R, L, true>, sm_rows);
+        if constexpr (APART) allow_smem<R>(k2_xfwd<R, L, true>, sm_rows);
         allow_smem<R>(k2_xfwd<R, L, false>, sm_rows);
         allow_smem<R>(k2_xinv<R, L>, sm_rows);
         allow_smem<R>(k2_cols<R, L, -1, true>, sm_cols);
@@ -1181,8 +1182,12 @@ spm_status apply_chunk_v2(const typename cplx_of<R>::type *xb, typename cplx_of<
         long rows = (long)nb * n2;
         // too few rows for a warp on every scheduler (4 x 152): the fields apart (n = 16 in
         // complex128: 20 us one after another)
-        if (rows * T < 32 * 4 * 152) launch_rows(k2_xfwd<R, L, true>, rows, 4, xb, m, p, W1, (int)rows, tw);
-        else launch_rows(k2_xfwd<R, L, false>, rows, 1, xb, m, p, W1, (int)rows, tw);
+        bool apart = false;
+        if constexpr (APART) {
+            apart = rows * T < 32 * 4 * 152;
+            if (apart) launch_rows(k2_xfwd<R, L, true>, rows, 4, xb, m, p, W1, (int)rows, tw);
+        }
+        if (!apart) launch_rows(k2_xfwd<R, L, false>, rows, 1, xb, m, p, W1, (int)rows, tw);
         mark();
         if constexpr (line_elems(L) == 8 && n % 2 == 0)
             launch_pdl(k2_cols2<R, L, -1, true>, dim3(L / TX, n / 2, nb * 4), dim3(THR), 2 * sm_cols, s, (const C *)W1,
