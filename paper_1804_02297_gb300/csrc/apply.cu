@@ -85,9 +85,10 @@ template <typename R, int L> struct tx_of {
 // complex64 only, where that choice is a bad one: k2_cols2 took 74 registers
 // (three blocks; 14.0 us against 12.1 with four), k2_zprod4 100 (still two
 // blocks, its loads in shorter batches; 30.7 us against 26.7 with 128).  One
-// application at n = 64: 70.9 us, 74.1 without.  The other lengths already
-// compile to these numbers, and a bound of one block there makes k2_cols2 keep
-// fewer blocks resident (L = 512: 946 us against 633).
+// application at n = 64: 70.9 us, 74.1 without.  From L = 256 on it already
+// compiles to these numbers, and a bound of one block there makes k2_cols2 keep
+// fewer blocks resident (L = 512: 946 us against 633); below L = 64 it
+// takes up to 70, not measured with a bound.
 template <typename R, int L> constexpr int pass_blocks(int regs)
 {
     return sizeof(R) == 4 && L == 128 ? 65536 / (regs * tx_of<R, L>::v * L / 8) : 0;
@@ -1677,13 +1678,13 @@ __global__ void __launch_bounds__(Q_THREADS) k_q(const float2 *__restrict__ v,
 }
 
 // Q in complex128: one thread per (point, output component), values and coefficients
-// straight from the caches.  Bound: the FP64 pipe (two lanes per SM, so a warp's FMA
-// takes 16 cycles): 972 n^3 FMAs, 6.3 us at n = 16 and 1.37 ms at n = 96.  Loads are
-// nearly free beside that, and what counts is that every SM gets the same share of full
-// warps: the 32 x 4 x 4 tiles of the complex64 kernel left one tile's work on each of 16
-// SMs at n = 16 (157 us; this kernel 17 us) and half-empty tiles elsewhere (n = 64: 600
-// against 416 us, n = 96: 1780 against 1395 us).  In complex64 the tiles win from n = 16
-// on (n = 64: 21 against 33 us) and the two are equal below.
+// straight from the caches.  Bound: the FP64 pipe (two lanes per SM: a warp's FMA takes 16
+// cycles of the SM's pipe, 64 of its scheduler's share): 972 n^3 FMAs, 6.3 us at n = 16 and
+// 1.37 ms at n = 96.  Loads are nearly free beside that, and what counts is that every SM
+// gets the same share of full warps: the 32 x 4 x 4 tiles of the complex64 kernel left one
+// tile's work on each of 16 SMs at n = 16 (157 us; this kernel 17 us) and half-empty tiles
+// elsewhere (n = 64: 600 against 416 us, n = 96: 1780 against 1395 us).  In complex64 the
+// tiles win from n = 16 on (n = 64: 21 against 33 us) and the two are equal below.
 // SPLIT = 3, for grids of fewer warps than schedulers: the three components d of a point
 // in three warps of a block, their sums joined through shared memory.
 template <typename C, int SPLIT>

@@ -81,8 +81,8 @@ spm_status spm_axpby_impl(int prec, long count, double a, const void *x, double 
 // is FP64: r = g - A x in complex128, stop when ||r_b||/||g_b|| <= tol for every
 // right-hand side b.  Each outer step runs one GMRES(restart) cycle on A d = r
 // (preconditioned residual), in complex128 (SPM_C128) or complex64 (SPM_C64,
-// SPM_MIXED) with FP64-accumulated dot products and FP64 Givens rotations on the
-// host, then x += d in FP64.  Right-hand sides are iterated together: every
+// SPM_MIXED) with FP64-accumulated dot products and FP64 Givens rotations, both on
+// the device, then x += d in FP64.  Right-hand sides are iterated together: every
 // operator and preconditioner application acts on the whole batch.
 namespace {
 

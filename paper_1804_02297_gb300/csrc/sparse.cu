@@ -534,8 +534,9 @@ inline unsigned blocks(long cnt, int t = 256) { return (unsigned)((cnt + t - 1) 
 //   forward, deepest level first:  [y; t] = G w_own,  Y_own = y,  W_bnd -= t
 //   backward, root first:          Y_own -= X Y_bnd
 // One launch per level and direction.  Every node's matrix (column-major, ld rows)
-// is cut into tiles of at most st_elems entries, copied to shared memory; a block of 256
-// threads owns one tile: thread t takes row t % nrow and the columns t / nrow + groups k,
+// is cut into tiles (of at most st_elems entries where they are copied to shared memory, 256
+// columns where they stream through registers, below); a block of 256 threads owns one tile:
+// thread t takes row t % nrow and the columns t / nrow + groups k,
 // groups = 256 / nrow, so that a tile of 49 rows keeps 245 threads busy.
 // Bound: complex64 by reading the factor; complex128 by the FP64 pipe (4 FMAs per
 // 16 bytes at 1.25 TFLOP/s: 2.5 TB/s); small grids by the 2 x levels dependent
@@ -609,7 +610,8 @@ template <int NB> struct TileAcc<float2, NB> {
 
 // Blocks per SM that the registers are held to.  complex64, one right-hand side: loads in
 // flight against blocks to overlap their starts and ends (3-D n = 32: four 392 us, five
-// 346, six 314, eight, which spill, 562; n = 64: 4.60, 3.94, 4.09, 6.46 ms).  Several wait on
+// 346, six 314, eight 562; n = 64: 4.60, 3.94, 4.09, 6.46 ms).  At six the streamed kernels
+// spill a few registers (one right-hand side 48 bytes a thread, two 104), at eight many.  Several wait on
 // shared memory between their packed FMAs and gain from warps (8 of them at n = 32: one
 // block 1050 us, two 686, three 606, four 586; 16, whose sums alone are 64 registers: one
 // 1599, two 1072, three 1585).  complex128 (2-D n = 239): one right-hand side four 342 us,
@@ -1109,7 +1111,7 @@ static spm_status factor_typed(const SparseSys &SY, NDFactor *F, bool half_store
     // (n = 64: 15 GB at 1536, 10 at 1024, at the same speed).  In 2-D the line stays at
     // 512: larger fronts would be faster batched too (n = 239: 137 -> 66 ms), but the
     // per-front path rounds differently, and 2-D factors have near-singular boxes often
-    // enough (one medium in ten at n = 239) that S^-1 moves by more than 1e-9.
+    // enough (one medium in twelve at n = 239) that S^-1 moves by 5e-9.
     std::vector<char> batched(NN, 0);
     for (const int fmax : BATCH_LINES) {
         if (fmax > (n3d == 1 ? 512 : most)) continue;
