@@ -616,19 +616,25 @@ template <int NB> struct TileAcc<float2, NB> {
 // block 1050 us, two 686, three 606, four 586; 16, whose sums alone are 64 registers: one
 // 1599, two 1072, three 1585).  complex128 (2-D n = 239): one right-hand side four 342 us,
 // five 312, six 294, eight 343; four 843, 840, 870, 884; eight 1802 with two, 1680 with four.
-template <typename C, int NB> constexpr int st_blocks()
+// Half storage streamed, one or two right-hand sides: eight, and no batches held in
+// registers: sixteen loads issued together straight into their FMAs (one right-hand side at
+// n = 64 2.49 ms; batches of eight at six blocks 3.34, of sixteen at four 3.54; two 2.59
+// against 3.71; n = 32 274 us against 283).
+template <typename C, typename S, int NB, bool STAGED> constexpr bool st_direct() { return !STAGED && sizeof(S) == 4 && NB <= 2; }
+template <typename C, typename S, int NB, bool STAGED> constexpr int st_blocks()
 {
+    if (st_direct<C, S, NB, STAGED>()) return 8;
     if (sizeof(C) == 16) return NB <= 2 ? 6 : (NB == 4 ? 5 : 4);
     return NB <= 2 ? 6 : (NB <= 8 ? 4 : 2);
 }
 
-template <typename C, typename S, int NB, bool FWD, bool STAGED>
-__global__ void __launch_bounds__(ST_THREADS, st_blocks<C, NB>()) k_nd_level(const S *__restrict__ M, const float *__restrict__ scales,
+template <typename C, typename S, int NB, bool FWD, bool STAGED, bool DIRECT = st_direct<C, S, NB, STAGED>()>
+__global__ void __launch_bounds__(ST_THREADS, st_blocks<C, S, NB, STAGED>()) k_nd_level(const S *__restrict__ M, const float *__restrict__ scales,
                                                          const SolveTile *__restrict__ tiles,
                                                          const int *__restrict__ bnd, C *W, C *Y, int nrhs, int tile_elems)
 {
     constexpr bool SCALED = !std::is_same<S, C>::value;
-    constexpr int UNR = STAGED ? 1 : (NB == 8 ? 4 : 8); // matrix entries a thread has in flight in registers
+    constexpr int UNR = STAGED || DIRECT ? 1 : (NB == 8 ? 4 : 8); // matrix entries a thread has in flight in registers
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S *ts = reinterpret_cast<S *>(smem_raw); // the tile, [ncol][nrow]
     C *xs = reinterpret_cast<C *>(smem_raw + (STAGED ? sizeof(S) * (size_t)tile_elems : 0)); // columns, then sums
@@ -652,7 +658,7 @@ __global__ void __launch_bounds__(ST_THREADS, st_blocks<C, NB>()) k_nd_level(con
         if (act)
             for (int c = g; c < tl.ncol; c += groups) cp_async<sizeof(S)>(&ts[c * tl.nrow + row], src + (long)c * tl.ld);
         cp_async_commit();
-    } else {
+    } else if constexpr (!DIRECT) {
         fetch(0);
     }
     pdl_wait_and_trigger();
@@ -660,7 +666,7 @@ __global__ void __launch_bounds__(ST_THREADS, st_blocks<C, NB>()) k_nd_level(con
         const int nb = min(NB, nrhs - b0);
         if (b0 > 0) {
             __syncthreads(); // the sums of the previous group have been read
-            if constexpr (!STAGED) fetch(0);
+            if constexpr (!STAGED && !DIRECT) fetch(0);
         }
         for (int i = threadIdx.x; i < tl.ncol * NB; i += ST_THREADS) {
             const int c = i / NB, b = i % NB;
@@ -679,6 +685,13 @@ __global__ void __launch_bounds__(ST_THREADS, st_blocks<C, NB>()) k_nd_level(con
             if (act) {
 #pragma unroll 4
                 for (int c = g; c < tl.ncol; c += groups) acc.mac(value_of(ts[c * tl.nrow + row]), xs + c * NB);
+            }
+        } else if constexpr (DIRECT) {
+            if (act) {
+                const S *q = src + (long)g * tl.ld;
+                const long step = (long)groups * tl.ld;
+#pragma unroll 16
+                for (int c = g; c < tl.ncol; c += groups, q += step) acc.mac(value_of(__ldcs(q)), xs + c * NB);
             }
         } else {
             for (int k0 = 0; k0 < steps; k0 += UNR) {
@@ -1421,7 +1434,7 @@ template <typename C, typename S, int NB, bool STAGED>
 static void launch_levels(NDFactor *F, const S *M, C *W, C *Y, int nrhs, cudaStream_t s)
 {
     // percent of 228 KB for the blocks that fit: NB x 256 sums and a reserved kilobyte each
-    constexpr int percent = st_blocks<C, NB>() * ((int)sizeof(C) * NB * ST_THREADS + 1024) / 2334 + 1;
+    constexpr int percent = st_blocks<C, S, NB, STAGED>() * ((int)sizeof(C) * NB * ST_THREADS + 1024) / 2334 + 1;
     static PerDevice<bool> opted;
     opted.get([]() -> std::optional<bool> { // a failure is the last error, which the solve checks after its launches
         if (opt_in(k_nd_level<C, S, NB, true, STAGED>, STAGED, percent) && opt_in(k_nd_level<C, S, NB, false, STAGED>, STAGED, percent))
